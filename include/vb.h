@@ -121,10 +121,11 @@ vb_status vb_profile_read(vb_ctx* ctx, float* ms, int64_t* launches);
  * and neighbours are ordered by (d2, j): distance first, then smaller index.
  * The search stages the points in a Morton order (of the coordinates when
  * m <= 4, of the projections on the cloud's 5 leading principal axes when
- * m > 4), prunes 64-point tiles by bounding boxes (in the FP32 search of a cloud
- * of more than 1,024 tiles, boxes of 64-tile super-tiles first; in the pipelined
- * 16-bit search, also balls about the box centres) and keeps the k + margin
- * nearest FP32 (or 16-bit) candidates per row;
+ * m > 4), prunes 64-point tiles by bounding boxes (boxes of 64-tile super-tiles
+ * first; in the pipelined 16-bit search, also balls about the box centres) and
+ * keeps the nearest FP32 (or 16-bit) candidates per row.  At m <= 8 and k <= 128
+ * one warp searches each pair of points and k + margin bounds the candidates that
+ * it rescores; otherwise one thread searches each point and keeps k + margin;
  * an FP64 rescoring with a proven FP32 error bound certifies every row, and
  * rows that fail it are recomputed by an exact FP64 radix selection.  The
  * output is therefore exact, identical to a brute-force FP64 search. */
@@ -169,8 +170,10 @@ typedef struct {
                                       cloud, e.g. ln(n_train / n_b) / d (NULL = none) */
     int32_t seed_tiles;      /* exact FP32 search: neighbouring tiles on each side of a query tile that are
                                 searched before any pruning (0 = enough to fill every heap) */
-    int32_t tc_variant;      /* 16-bit tiles: VB_TC_AUTO (FP16: pipelined when its shared memory fits, else
-                                staged; BF16: staged), VB_TC_STAGED or VB_TC_PIPELINED (VB_ERR_UNSUPPORTED
+    int32_t tc_variant;      /* 16-bit tiles: VB_TC_AUTO (m <= 4 and k <= 128, without diagnostic output: the
+                                FP32 warp search, faster there than either tensor-core kernel, whose one MMA
+                                step of K = 16 holds 4 coordinates; else FP16: pipelined when its shared memory
+                                fits, else staged; BF16: staged), VB_TC_STAGED or VB_TC_PIPELINED (VB_ERR_UNSUPPORTED
                                 when k + margin and m leave no room for two ring slots).  The pipelined
                                 kernel centres its operands on the whole cloud, not on each query tile,
                                 so its 16-bit error band is wider: exact either way, but with BF16 many

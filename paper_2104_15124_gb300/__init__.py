@@ -273,7 +273,8 @@ def knn(x: torch.Tensor, k: int, margin: int = 16, prune: bool = True, radius: t
     """Exact kNN (vb_knn): returns (nbr int32 [n, k], nbr_d2 fp64 [n, k]).  With `radius` (per-point
     guess of the k-th neighbour distance) or a learned `mlp`, the radius-first search runs;
     tensor_cores = "fp16" or "bf16" computes its distance tiles on the tensor cores, with the
-    kernel tc_variant = "auto", "staged" or "pipelined" (VB_TC_*); seed_tiles and heap_keys
+    kernel tc_variant = "auto" (at m <= 4 the FP32 warp search, which is faster there), "staged" or
+    "pipelined" (VB_TC_*); seed_tiles and heap_keys
     ("compact" or "full") and curve ("auto": Hilbert order at 2 <= m <= 4, or "morton") as in
     vb_knn_params.  debug=True (16-bit tiles) also returns the
     candidates each row kept and their 16-bit tile distances before rescoring:

@@ -24,6 +24,7 @@
 //       Uncertified rows (ties, duplicates) are recomputed by an exact FP64
 //       radix selection over all points.
 #include "vb_internal.cuh"
+#include "knn.cuh"
 #include "tc.cuh"
 
 #include <cuda_bf16.h>
@@ -34,7 +35,6 @@
 
 namespace vb {
 
-constexpr int TILE = 64;            // points per query tile and per candidate tile
 constexpr int RADIX_T = 256;        // threads of the radix kernels
 constexpr int RADIX_ITEMS = 2048;   // keys per radix block (8 rounds of 256)
 constexpr int USCAN_T = 1024, USCAN_ITEMS = 8, USCAN_CHUNK = USCAN_T * USCAN_ITEMS;   // histogram scan
@@ -642,72 +642,6 @@ __device__ __forceinline__ double canon_d2_64(const double* a, const double* __r
     return acc;
 }
 
-// The same for a query held in registers (q[0..MP)) and a 16-byte aligned candidate row.
-template <int MP>
-__device__ __forceinline__ double canon_d2_q64(const double* q, const double* __restrict__ c, int m)
-{
-    double cv[MP];
-#pragma unroll
-    for (int r2 = 0; r2 < MP / 2; ++r2) {
-        const double2 v = *(const double2*)(c + 2 * r2);
-        cv[2 * r2] = v.x;
-        cv[2 * r2 + 1] = v.y;
-    }
-    double acc = 0.0;
-#pragma unroll
-    for (int r = 0; r < MP; ++r) {
-        if (r < m) {
-            const double dl = __dsub_rn(q[r], cv[r]);
-            const double sq = __dmul_rn(dl, dl);
-            acc = r == 0 ? sq : __dadd_rn(acc, sq);
-        }
-    }
-    return acc;
-}
-
-struct TileArgs {
-    const float* xs;
-    const double* xs64;   // FP64 copies of xs (exact), for the FP64 rescoring
-    const float* tlo;
-    const float* thi;
-    const float* slo;     // boxes of super-tiles (64 consecutive tiles; FP32 search)
-    const float* shi;
-    const uint32_t* perm;
-    int64_t n;
-    int64_t ntiles;
-    int m, k, L, prune, nseed;
-    float lb_factor;     // 1 - 4 (m + 2) 2^-24, applied rounding down
-    float band;          // 1 + 4 (m + 2) 2^-24: FP32 distances closer than this may swap in FP64
-    double cert_factor;  // 1 - 2 (m + 2) 2^-24
-    int32_t* nbr;
-    double* nbr_d2;
-    int* fb_list;
-    int* fb_count;
-    int* work;           // next query tile (persistent grid)
-    const int* tile_list;   // optional list of query tiles to process (else all tiles)
-    const int* tile_count;  // its length (device)
-    const float* r2;        // radius search: per sorted point, squared radius bound
-    float r2_scale;         // radius search: factor on r2 for this pass
-    int count_retries;      // radius search: count the tiles this pass hands on (last pass only)
-    int cap;                // radius search: candidates kept per query
-    int* fail_flag;         // radius search: per query tile, set once it joins fail_list
-    int* fail_list;
-    int* fail_count;
-    Clouds cl;              // batched build: queries only take candidates from their own cloud
-    DevReport* rep;
-    // pipelined 16-bit search
-    const unsigned char* blk;   // tile blocks (operand image + norms), tcp_blk_bytes(kp) each
-    int kp;                     // K: m padded to 16
-    int stages;                 // ring slots of staged tile blocks
-    uint32_t* lbw;              // per CTA scratch: ntiles box bounds
-    uint64_t* tlist;            // per CTA scratch: ntiles (bound, tile) keys in bound order
-    uint4* lbs;                 // per CTA scratch: ntiles bounds of the four 32-query groups
-    const float* trad;          // per tile: radius of its ball about the box centre (pipelined search)
-    uint64_t* hdump;            // pipelined search: heaps handed to its row finish ([L][128] per query tile)
-    float* dbg_d2;              // diagnostic: kept 16-bit distances per row ([n][L], original order)
-    int32_t* dbg_idx;           // their original indices
-};
-
 constexpr int IB = 8;         // candidate distances computed per batch before any insertion
 constexpr int SCAP = 256;     // candidate tiles per sorted chunk
 constexpr int FLAT_SUPERS = 16;   // up to this many super-tiles (64 tiles each) in range: one-level scan
@@ -810,18 +744,6 @@ template <> struct KeyOps<true> {
         return ((dbits >> 13) << 14) | ((uint32_t)vis << 6) | (uint32_t)c;
     }
 };
-
-template <int MP>
-__device__ __forceinline__ float point_box_lb(const float* q, const float* lo, const float* hi)
-{
-    float acc = 0.f;
-#pragma unroll
-    for (int r = 0; r < MP; ++r) {
-        float g = fmaxf(fmaxf(lo[r] - q[r], q[r] - hi[r]), 0.f);
-        acc = fmaf(g, g, acc);
-    }
-    return acc;
-}
 
 // Orders the candidates of one query and writes its row (step a5).  arr[0..size)
 // holds keys (FP32 distance bits << 32 | sorted position), column t of a [.][TILE]
@@ -3037,7 +2959,10 @@ vb_status knn_run(Ctx* ctx, const float* x, int64_t n, int32_t m, const vb_knn_p
     const bool tensor = p->precision == VB_PREC_BF16 || p->precision == VB_PREC_FP16;
     // the tiles a radius-first or 16-bit first pass hands back are searched with compact keys
     // before the full-key search takes what is left
-    const bool compact_retry = (radius_first || tensor) && p->heap_keys != VB_KEYS_FULL && mp <= 16;
+    // m <= 8: the warp search, also for 16-bit requests at m <= 4 that name no kernel and want no diagnostic
+    const bool warp_search = warp_search_takes(mp, p) &&
+                             (!tensor || (mp == 4 && p->tc_variant == VB_TC_AUTO && !a.dbg_d2));
+    const bool compact_retry = (radius_first || tensor) && p->heap_keys != VB_KEYS_FULL && mp <= 16 && !warp_search;
     int launches = 0;
     if (radius_first || tensor) {
         if (radius_first) {
@@ -3064,7 +2989,10 @@ vb_status knn_run(Ctx* ctx, const float* x, int64_t n, int32_t m, const vb_knn_p
         a.fail_flag = w.fail_flag;
         a.fail_list = w.fail_list;
         a.fail_count = w.fb_count + 3;
-        if (tensor) {
+        if (warp_search) {
+            launches += 1;
+            st = launch_warp_search(a, mp, s);
+        } else if (tensor) {
             a.cap = a.L;
             st = VB_ERR_UNSUPPORTED;
             // automatic choice: pipelined for FP16; BF16's 8-bit significand needs the staged kernel's
@@ -3143,13 +3071,14 @@ vb_status knn_run(Ctx* ctx, const float* x, int64_t n, int32_t m, const vb_knn_p
         a.fail_list = w.fail_list;
         a.fail_count = w.fb_count + 3;
         launches += 1;
-        switch (mp) {
-            case 4: st = launch_tile<4, true>(a, s); break;
-            case 8: st = launch_tile<8, true>(a, s); break;
-            case 16: st = launch_tile<16, true>(a, s); break;
-            case 32: st = launch_tile<32, true>(a, s); break;
-            case 64: st = launch_tile<64, true>(a, s); break;
-            default: st = launch_tile<128, true>(a, s); break;
+        if (warp_search) {
+            st = launch_warp_search(a, mp, s);
+        } else {
+            switch (mp) {
+                case 4: st = launch_tile<4, true>(a, s); break;
+                case 8: st = launch_tile<8, true>(a, s); break;
+                default: st = launch_tile<16, true>(a, s); break;
+            }
         }
         if (st != VB_OK) return st;
         a.work = w.fb_count + 2;

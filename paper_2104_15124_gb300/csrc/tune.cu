@@ -68,9 +68,10 @@ extern "C" vb_status vb_knn_autotune(vb_ctx* ctx, const float* x, int64_t n, int
     const int margins[] = {2, 4, 8, 16, 32};
     const int seeds_fp32[] = {1, 2, 3};
     const int seeds_tc[] = {0};
-    // 16-bit tiles: both kernels; the FP32 search has one
-    const int variants_tc[] = {VB_TC_PIPELINED, VB_TC_STAGED};
-    const int nv = fp32 ? 1 : 2;
+    // 16-bit requests: both tensor-core kernels and, at m <= 4, the automatic choice (the warp search);
+    // the FP32 search has one
+    const int variants_tc[] = {VB_TC_PIPELINED, VB_TC_STAGED, VB_TC_AUTO};
+    const int nv = fp32 ? 1 : m <= 4 ? 3 : 2;
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess) return VB_ERR_CUDA;
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return VB_ERR_CUDA; }
