@@ -27,8 +27,24 @@ struct DeviceGuard {
 
 Ctx* C(vb_ctx* c) { return reinterpret_cast<Ctx*>(c); }
 
-// A batched build keeps the cloud of every point at the front of the workspace.
-size_t cloud_id_bytes(int64_t n, int B) { return B > 1 ? (((size_t)n * sizeof(int32_t) + 255) & ~(size_t)255) : 0; }
+// The front of a build's workspace: what its passes share, and the cloud of every point of a batch.
+struct Front {
+    BuildAux aux;
+    int32_t* id = nullptr;
+};
+size_t front_plan(void* ws, int64_t n, int B, Front* f)
+{
+    Carve c(ws);
+    Front t;
+    t.aux.ib = c.take<float>(n);
+    t.aux.iP = c.take<float>(n);
+    t.aux.pv = c.take<PointOp>(n);
+    t.aux.part_den = c.take<double>(pair_slots(B));
+    if (B > 1) t.id = c.take<int32_t>(n);
+    c.take<char>(0);   // round up: the stages' workspace follows, 256-byte aligned
+    if (f) *f = t;
+    return c.off;
+}
 
 size_t build_ws(int64_t n, int32_t m, const vb_build_params* p, int B = 1)
 {
@@ -36,7 +52,7 @@ size_t build_ws(int64_t n, int32_t m, const vb_build_params* p, int B = 1)
     size_t knn = knn_plan(c, n, m, &p->knn, nullptr);
     size_t s = std::max({knn, graph_plan_bytes(n, p->knn.k), sweep_ws_bytes(n, B), density_ws_bytes(n, B),
                          centre_ws_bytes(n, B), kernel_csr_ws_bytes(n, B)});
-    return s + cloud_id_bytes(n, B);
+    return s + front_plan(nullptr, n, B, nullptr);
 }
 
 __global__ void cloud_id_kernel(const int64_t* __restrict__ ptr, int B, int64_t n, int32_t* id)
@@ -53,37 +69,43 @@ vb_status build_run(Ctx* c, const float* x, int64_t n, int32_t m, const vb_build
     const int32_t k_bw = p->k_bw > 0 ? p->k_bw : k;
     if (k_bw > k) return VB_ERR_ARG;
     if (!ws || ws_bytes < build_ws(n, m, p, cl.B)) return VB_ERR_WORKSPACE;
+    Front f;
+    const size_t off = front_plan(ws, n, cl.B, &f);
+    ws = (char*)ws + off;
+    ws_bytes -= off;
     if (cl.B > 1) {
-        int32_t* id = (int32_t*)ws;
-        const size_t off = cloud_id_bytes(n, cl.B);
-        cloud_id_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(cl.ptr, cl.B, n, id);
+        cloud_id_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(cl.ptr, cl.B, n, f.id);
         c->launches += 1;
-        cl.id = id;
-        ws = (char*)ws + off;
-        ws_bytes -= off;
+        cl.id = f.id;
     }
     vb_status st = knn_run(c, x, n, m, &p->knn, o->nbr, o->nbr_d2, ws, ws_bytes, cl);
     if (st) return st;
     st = graph_run(c, n, k, o->nbr, o->nbr_d2, o->row_ptr, o->col, o->ed2, o->cap, o->nnz, ws, ws_bytes);
     if (st) return st;
-    st = bandwidth_run(c, n, k, k_bw, o->nbr_d2, o->b);
+    st = bandwidth_run(c, n, k, k_bw, o->nbr_d2, o->b, f.aux.ib);
     if (st) return st;
     vb_graph gr{n, o->row_ptr, o->col, o->ed2};
+    f.aux.t = o->val;   // free until L-hat is written
+    st = pair_run(c, &gr, f.aux.ib, f.aux.t, f.aux.part_den, cl);
+    if (st) return st;
+    mark(c, VB_STAGE_BANDWIDTH, 1);   // the products of b belong to its stage
     if (!p->pin_eps) {
         st = sweep_run(c, &gr, o->b, 1.0, nullptr, p->xi_lo, p->xi_hi, p->dxi, 1, o->eps2_den, o->chi_den, o->dim_den,
-                       ws, ws_bytes, cl);
+                       ws, ws_bytes, cl, f.aux.ib, f.aux.t);
         if (st) return st;
     }
-    st = density_run(c, &gr, o->b, o->eps2_den, p->op.d, p->op.beta, o->psi, o->P, ws, ws_bytes, cl);
+    st = density_run(c, &gr, o->b, o->eps2_den, p->op.d, p->op.beta, o->psi, o->P, ws, ws_bytes, cl, 8,
+                     f.aux);
     if (st) return st;
-    st = centre_run(c, &gr, o->b, o->P, o->xi_c, ws, ws_bytes, cl);
+    st = centre_run(c, &gr, o->b, o->P, o->xi_c, ws, ws_bytes, cl, f.aux);
     if (st) return st;
     if (!p->pin_eps) {
         st = sweep_run(c, &gr, o->P, 4.0, o->xi_c, p->xi_lo, p->xi_hi, p->dxi, 2, o->eps2_op, o->chi_op, o->dim_op, ws,
-                       ws_bytes, cl);
+                       ws_bytes, cl, f.aux.iP, f.aux.t);
         if (st) return st;
     }
-    return kernel_csr_run(c, &gr, o->psi, o->P, &p->op, o->eps2_op, o->val, o->q, o->D, o->S, ws, ws_bytes, cl);
+    return kernel_csr_run(c, &gr, o->psi, o->P, &p->op, o->eps2_op, o->val, o->q, o->D, o->S, ws, ws_bytes, cl, 8,
+                          f.aux);
 }
 
 }  // namespace

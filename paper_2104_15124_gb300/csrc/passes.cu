@@ -64,23 +64,7 @@ struct RowGroup {
     }
 };
 
-// A lane's next UNR entries of a row (stride LPR): their column and squared distance
-// loaded together (column -1 past the row's end), so the gathers that follow are all in
-// flight at once; the lane still adds its entries in increasing order, as a plain loop would.
-constexpr int UNR = 4;
-template <int LPR>
-__device__ __forceinline__ void load_entries(const int32_t* __restrict__ col, const float* __restrict__ ed2,
-                                             int64_t e0, int64_t re, int32_t* jj, float* xx)
-{
-#pragma unroll
-    for (int u = 0; u < UNR; ++u) {
-        const int64_t e = e0 + (int64_t)u * LPR;
-        const bool in = e < re;
-        jj[u] = in ? col[e] : -1;
-        xx[u] = in ? ed2[e] : 0.f;
-    }
-}
-
+constexpr int UNR = 4;   // entries a lane loads together, so that the gathers that follow are all in flight at once
 // The lane's quad of consecutive entries b0 .. b0 + 3 (b0 a multiple of 4) of the row [rb, re):
 // one 16-byte load of the columns and one of the squared distances when the quad lies inside
 // the row and the arrays are 16-byte aligned, else four masked loads (column -1 outside the
@@ -239,7 +223,9 @@ __global__ void __launch_bounds__(kRowThreads) sweep_kernel(const int64_t* __res
 // r_{g-4} = 2 r_g, so exp(-t r_{g-4}) = exp(-t r_g)^2.  Each of the four chains
 // g = 56 - c, 52 - c, ... takes an ex2 at every fourth step and squares in
 // between (relative error at most 8x that of ex2, about 2e-6), which moves the
-// pass from the SFU to the FMA pipe.  A warp owns a contiguous range of rows and
+// pass from the SFU to the FMA pipe.  Two chains share every multiplication and addition (packed
+// FP32x2, the scalar form's rounding: the same bits), which halves the instructions of a pass that
+// is bound by issue.  A warp owns a contiguous range of rows and
 // its lanes stride that range's entries, so every lane stays busy whatever the
 // row lengths; the row of an entry is tracked by a cursor per lane.
 constexpr int G57 = 57;
@@ -286,10 +272,14 @@ __device__ __forceinline__ void warp_reduce_scatter64(const float (&a)[G57], flo
     s1 = f[1];
 }
 
+// READY: the entries' t = ed2 (r_i r_j) are in tt (pair_kernel: the same products, so the same bits),
+// and the pass is a plain stream of them.
+template <bool READY>
 __global__ void __launch_bounds__(kRowThreads, 2) sweep57_kernel(const int64_t* __restrict__ row_ptr,
                                                             const int32_t* __restrict__ col,
                                                             const float* __restrict__ ed2, int64_t n,
                                                             const float* __restrict__ irho,
+                                                            const float* __restrict__ tt,
                                                             const double* __restrict__ xi_c_dev, double scale,
                                                             SweepConst sc, Clouds cl, double* partial)
 {
@@ -300,7 +290,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) sweep57_kernel(const int64_t* 
     const int64_t r0 = min(n, (int64_t)blockIdx.x * per), r1 = min(n, r0 + per);
     if (r0 >= r1) return;
     const int cf = cloud_of(cl.ptr, cl.B, r0), cla = cloud_of(cl.ptr, cl.B, r1 - 1);
-    float acc[G57];
+    float2 acc[G57 / 2];   // grid points 56 - 2 q and 55 - 2 q
+    float acc0;            // grid point 0
     for (int cb = cf; cb <= cla; ++cb) {
         for (int i = threadIdx.x; i < WARPS * G57; i += blockDim.x) (&wacc[0][0])[i] = 0.0;
         if (threadIdx.x == 0) {
@@ -313,65 +304,95 @@ __global__ void __launch_bounds__(kRowThreads, 2) sweep57_kernel(const int64_t* 
         const int64_t pw = (s1 - s0 + WARPS - 1) / WARPS;
         const int64_t a0 = min(s1, s0 + w * pw), a1 = min(s1, a0 + pw);
         const int64_t e0 = row_ptr[a0], e1 = row_ptr[a1];
+        auto clear = [&]() {
 #pragma unroll
-        for (int g = 0; g < G57; ++g) acc[g] = 0.f;
+            for (int q = 0; q < G57 / 2; ++q) acc[q] = make_float2(0.f, 0.f);
+            acc0 = 0.f;
+        };
+        clear();
         double dacc0 = 0.0, dacc1 = 0.0;   // this lane's share of the warp's totals: slots 2 lane, 2 lane + 1
         auto flush = [&]() {
-            float s0, s1;
-            warp_reduce_scatter64(acc, s0, s1);
+            float a[G57], s0, s1;
+            a[0] = acc0;
+#pragma unroll
+            for (int q = 0; q < G57 / 2; ++q) {
+                a[G57 - 1 - 2 * q] = acc[q].x;
+                a[G57 - 2 - 2 * q] = acc[q].y;
+            }
+            warp_reduce_scatter64(a, s0, s1);
             dacc0 += (double)s0;
             dacc1 += (double)s1;
-#pragma unroll
-            for (int g = 0; g < G57; ++g) acc[g] = 0.f;
+            clear();
         };
-        int64_t i = a0;
-        int64_t inext = row_ptr[min(a0 + 1, n)];
-        float ri = a0 < n ? irho[a0] : 0.f;
-        int64_t inext2 = row_ptr[min(a0 + 2, n)];   // the next row's end and bandwidth, loaded a row ahead
-        float ri_next = irho[min(a0 + 1, n - 1)];
         int since = 0;
-        // software pipeline: the column and squared distance of the entry three chunks ahead and
-        // the bandwidth gather of the entry two chunks ahead are in flight while this chunk's 57
-        // kernel values are formed (column -1: past the warp's range); the row cursor keeps the
-        // next row's end and bandwidth loaded a row ahead
-        int32_t j0 = -1, j1 = -1, j2 = -1;
-        float x0 = 0.f, x1 = 0.f, x2 = 0.f;
-        if (e0 + lane < e1) { j0 = col[e0 + lane]; x0 = ed2[e0 + lane]; }
-        if (e0 + 32 + lane < e1) { j1 = col[e0 + 32 + lane]; x1 = ed2[e0 + 32 + lane]; }
-        if (e0 + 64 + lane < e1) { j2 = col[e0 + 64 + lane]; x2 = ed2[e0 + 64 + lane]; }
-        float rj0 = j0 >= 0 ? irho[j0] : 0.f;
-        float rj1 = j1 >= 0 ? irho[j1] : 0.f;
-        for (int64_t eb = e0; eb < e1; eb += 32) {
-            const int64_t e = eb + lane;
-            int32_t j3 = -1;
-            float x3 = 0.f;
-            if (e + 96 < e1) { j3 = col[e + 96]; x3 = ed2[e + 96]; }
-            const float rj2 = j2 >= 0 ? irho[j2] : 0.f;
-            float u = INFINITY;
-            if (e < e1) {
-                while (inext <= e) {
-                    ++i;
-                    inext = inext2;
-                    ri = ri_next;
-                    inext2 = row_ptr[min(i + 2, n)];
-                    ri_next = irho[min(i + 1, n - 1)];
-                }
-                if (j0 != i) u = x0 * (ri * rj0) * c0;
-            }
-            j0 = j1; x0 = x1; rj0 = rj1;
-            j1 = j2; x1 = x2; rj1 = rj2;
-            j2 = j3; x2 = x3;
-            float prev[4];
+        auto fold = [&](float u) {   // the 57 kernel values of one entry per lane
+            float2 prev[2];
 #pragma unroll
-            for (int g = G57 - 1; g >= 0; --g) {
-                const int c = (G57 - 1 - g) & 3, step = (G57 - 1 - g) >> 2;
-                const float v = (step & 3) == 0 ? ex2_approx(u * sc.negr[g]) : prev[c] * prev[c];
-                prev[c] = v;
-                acc[g] += v;
+            for (int q = 0; q < G57 / 2; ++q) {
+                const int c = q & 1, step = q >> 1, g = G57 - 1 - 2 * q;
+                if ((step & 3) == 0) prev[c] = make_float2(ex2_approx(u * sc.negr[g]), ex2_approx(u * sc.negr[g - 1]));
+                else prev[c] = __fmul2_rn(prev[c], prev[c]);
+                acc[q] = __fadd2_rn(acc[q], prev[c]);
             }
+            acc0 += prev[0].x * prev[0].x;   // step 14 of the first chain
             if (++since == 32) {
                 since = 0;
                 flush();
+            }
+        };
+        if constexpr (READY) {
+            constexpr int AHEAD = 4;   // chunks of 32 entries in flight
+            float x[AHEAD];
+#pragma unroll
+            for (int h = 0; h < AHEAD; ++h) x[h] = e0 + 32 * h + lane < e1 ? tt[e0 + 32 * h + lane] : -0.f;
+            for (int64_t eb = e0; eb < e1; eb += 32 * AHEAD) {
+#pragma unroll
+                for (int h = 0; h < AHEAD; ++h) {
+                    if (eb + 32 * h >= e1) break;
+                    const float t = x[h];
+                    const int64_t e = eb + 32 * (AHEAD + h) + lane;
+                    x[h] = e < e1 ? tt[e] : -0.f;
+                    fold(signbit(t) ? INFINITY : t * c0);
+                }
+            }
+        } else {
+            int64_t i = a0;
+            int64_t inext = row_ptr[min(a0 + 1, n)];
+            float ri = a0 < n ? irho[a0] : 0.f;
+            int64_t inext2 = row_ptr[min(a0 + 2, n)];   // the next row's end and bandwidth, loaded a row ahead
+            float ri_next = irho[min(a0 + 1, n - 1)];
+            // software pipeline: the column and squared distance of the entry three chunks ahead and
+            // the bandwidth gather of the entry two chunks ahead are in flight while this chunk's 57
+            // kernel values are formed (column -1: past the warp's range); the row cursor keeps the
+            // next row's end and bandwidth loaded a row ahead
+            int32_t j0 = -1, j1 = -1, j2 = -1;
+            float x0 = 0.f, x1 = 0.f, x2 = 0.f;
+            if (e0 + lane < e1) { j0 = col[e0 + lane]; x0 = ed2[e0 + lane]; }
+            if (e0 + 32 + lane < e1) { j1 = col[e0 + 32 + lane]; x1 = ed2[e0 + 32 + lane]; }
+            if (e0 + 64 + lane < e1) { j2 = col[e0 + 64 + lane]; x2 = ed2[e0 + 64 + lane]; }
+            float rj0 = j0 >= 0 ? irho[j0] : 0.f;
+            float rj1 = j1 >= 0 ? irho[j1] : 0.f;
+            for (int64_t eb = e0; eb < e1; eb += 32) {
+                const int64_t e = eb + lane;
+                int32_t j3 = -1;
+                float x3 = 0.f;
+                if (e + 96 < e1) { j3 = col[e + 96]; x3 = ed2[e + 96]; }
+                const float rj2 = j2 >= 0 ? irho[j2] : 0.f;
+                float u = INFINITY;
+                if (e < e1) {
+                    while (inext <= e) {
+                        ++i;
+                        inext = inext2;
+                        ri = ri_next;
+                        inext2 = row_ptr[min(i + 2, n)];
+                        ri_next = irho[min(i + 1, n - 1)];
+                    }
+                    if (j0 != i) u = x0 * (ri * rj0) * c0;
+                }
+                j0 = j1; x0 = x1; rj0 = rj1;
+                j1 = j2; x1 = x2; rj1 = rj2;
+                j2 = j3; x2 = x3;
+                fold(u);
             }
         }
         flush();
@@ -440,7 +461,7 @@ size_t sweep_ws_bytes(int64_t n, int B)
 
 vb_status sweep_run(Ctx* ctx, const vb_graph* g, const double* rho, double scale, const double* xi_c_dev,
                     double xi_lo, double xi_hi, double dxi, int warn_bit, double* eps2, double* chi, double* dim,
-                    void* ws, size_t ws_bytes, Clouds cl)
+                    void* ws, size_t ws_bytes, Clouds cl, const float* irho_ready, const float* t_ready)
 {
     if (!g || !g->row_ptr || !g->col || !g->ed2 || g->n < 1 || !rho || !eps2 || !chi || !dim) return VB_ERR_ARG;
     if (!(dxi > 0) || !(scale > 0) || cl.B < 1 || (cl.B > 1 && !cl.ptr)) return VB_ERR_ARG;
@@ -454,18 +475,26 @@ vb_status sweep_run(Ctx* ctx, const vb_graph* g, const double* rho, double scale
     for (int h = 0; h < kMaxGrid; ++h) sc.negr[h] = h < G ? -(float)std::exp2(-(xi_lo + h * dxi)) : 0.f;
     cudaStream_t s = ctx->stream;
     const int stage = warn_bit == 2 ? VB_STAGE_SWEEP_OPERATOR : VB_STAGE_SWEEP_DENSITY;
-    recip_f32_kernel<<<(unsigned)((g->n + 255) / 256), 256, 0, s>>>(rho, g->n, 1.f, irho);
+    if (irho_ready) {
+        irho = const_cast<float*>(irho_ready);
+    } else {
+        recip_f32_kernel<<<(unsigned)((g->n + 255) / 256), 256, 0, s>>>(rho, g->n, 1.f, irho);
+        ctx->launches += 1;
+    }
     mark(ctx, stage, 0);
-    if (G == G57 && dxi == 0.25)
-        sweep57_kernel<<<kSweepBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, irho, xi_c_dev, scale, sc,
-                                                          cl, partial);
+    if (G == G57 && dxi == 0.25 && t_ready)
+        sweep57_kernel<true><<<kSweepBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, irho, t_ready, xi_c_dev,
+                                                                scale, sc, cl, partial);
+    else if (G == G57 && dxi == 0.25)
+        sweep57_kernel<false><<<kSweepBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, irho, nullptr, xi_c_dev,
+                                                                 scale, sc, cl, partial);
     else
         sweep_kernel<<<kSweepBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, irho, xi_c_dev, scale, G, sc,
                                                         cl, partial);
     mark(ctx, stage, 1);
     sweep_finish_kernel<<<(unsigned)cl.B, 1024, 0, s>>>(partial, kSweepBlocks, G, g->n, cl, xi_lo, dxi, xi_c_dev,
                                                         warn_bit, eps2, chi, dim, ctx->rep);
-    ctx->launches += 3;
+    ctx->launches += 2;
     return last_launch();
 }
 
@@ -477,29 +506,47 @@ __global__ void density_const_kernel(const double* __restrict__ eps2, int B, flo
     if (b < B) c[b] = (float)(1.4426950408889634 / eps2[b]);
 }
 
-template <int LPR>
+// READY: the products t are in tt (pair_kernel), and the rows are a stream (0.30 -> 0.10 ms at 1M points).
+template <int LPR, bool READY>
 __global__ void __launch_bounds__(kRowThreads) density_kernel(const int64_t* __restrict__ row_ptr,
                                                             const int32_t* __restrict__ col,
                                                             const float* __restrict__ ed2, int64_t n,
                                                             const float* __restrict__ ib,
+                                                            const float* __restrict__ tt,
                                                             const float* __restrict__ cden, Clouds cl, double* psi)
 {
     RowGroup<LPR> it;
-    const bool vec = aligned16(col, ed2);
+    const bool vec = READY ? aligned16(tt, tt) : aligned16(col, ed2);
     for (int64_t b0 = it.base; b0 < n; b0 += it.step) {
         const int64_t i = b0 + it.grp;
         const bool ok = i < n;
         const float c = ok ? cden[cloud_id(cl, i)] : 0.f;
         const int64_t rb = ok ? row_ptr[i] : 0, re = ok ? row_ptr[i + 1] : 0;
-        const float bi = ok ? ib[i] : 0.f;
         float s = 0.f;
-        for (int64_t e0 = quad_start(rb, it.sub); e0 < re; e0 += 4 * LPR) {
-            int32_t jj[UNR];
-            float xx[UNR];
-            load_quad(col, ed2, vec, e0, rb, re, jj, xx);
+        if constexpr (READY) {
+            for (int64_t e0 = quad_start(rb, it.sub); e0 < re; e0 += 4 * LPR) {
+                if (vec && e0 >= rb && e0 + 3 < re) {
+                    const float4 t4 = *(const float4*)(tt + e0);
+                    s += ex2_approx(-t4.x * c);
+                    s += ex2_approx(-t4.y * c);
+                    s += ex2_approx(-t4.z * c);
+                    s += ex2_approx(-t4.w * c);
+                } else {
 #pragma unroll
-            for (int u = 0; u < UNR; ++u)
-                if (jj[u] >= 0) s += ex2_approx(-(xx[u] * (bi * ib[jj[u]])) * c);
+                    for (int u = 0; u < 4; ++u)
+                        if (e0 + u >= rb && e0 + u < re) s += ex2_approx(-tt[e0 + u] * c);
+                }
+            }
+        } else {
+            const float bi = ok ? ib[i] : 0.f;
+            for (int64_t e0 = quad_start(rb, it.sub); e0 < re; e0 += 4 * LPR) {
+                int32_t jj[UNR];
+                float xx[UNR];
+                load_quad(col, ed2, vec, e0, rb, re, jj, xx);
+#pragma unroll
+                for (int u = 0; u < UNR; ++u)
+                    if (jj[u] >= 0) s += ex2_approx(-(xx[u] * (bi * ib[jj[u]])) * c);
+            }
         }
         const float tot = RowGroup<LPR>::sum(s);
         if (ok && it.sub == 0) psi[i] = (double)tot;
@@ -511,7 +558,8 @@ __global__ void __launch_bounds__(kRowThreads) density_kernel(const int64_t* __r
 // every operator-kernel exponent, so its error is multiplied by exponents of up to
 // about 60 in the smallest stored entries.
 __global__ void density_finish_kernel(const double* __restrict__ b, const double* __restrict__ eps2_dev, int64_t n,
-                                      Clouds cl, double d, double beta, double* psi, double* P)
+                                      Clouds cl, double d, double beta, double* psi, double* P,
+                                      float* iP, PointOp* pv)
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -524,7 +572,15 @@ __global__ void density_finish_kernel(const double* __restrict__ b, const double
     const double w = nb * (e == 1.0 ? x : e == 0.5 ? sqrt(x) : e == 2.5 ? x * x * sqrt(x) : pow(x, e));
     const double ps = psi[i] / w;
     psi[i] = ps;
-    P[i] = beta == -0.25 ? 1.0 / sqrt(sqrt(ps)) : pow(ps, beta);
+    const double p = beta == -0.25 ? 1.0 / sqrt(sqrt(ps)) : pow(ps, beta);
+    P[i] = p;
+    if (iP) {   // a build: the reciprocals that the passes to come gather, one FP64 division for all of them
+        const double r = 1.0 / p;
+        const float h = (float)r;
+        iP[i] = h;
+        pv[i].iPh = h;
+        pv[i].iPl = (float)(r - (double)h);
+    }
 }
 
 size_t density_ws_bytes(int64_t n, int B)
@@ -536,7 +592,7 @@ size_t density_ws_bytes(int64_t n, int B)
 }
 
 vb_status density_run(Ctx* ctx, const vb_graph* g, const double* b, const double* eps2_dev, double d, double beta,
-                      double* psi, double* P, void* ws, size_t ws_bytes, Clouds cl, int lpr)
+                      double* psi, double* P, void* ws, size_t ws_bytes, Clouds cl, int lpr, const BuildAux& aux)
 {
     if (!g || !g->row_ptr || !b || !eps2_dev || !psi || !P || !(d > 0)) return VB_ERR_ARG;
     if (cl.B < 1 || (cl.B > 1 && !cl.ptr)) return VB_ERR_ARG;
@@ -546,126 +602,172 @@ vb_status density_run(Ctx* ctx, const vb_graph* g, const double* b, const double
     if (!ws || ws_bytes < c.off) return VB_ERR_WORKSPACE;
     cudaStream_t s = ctx->stream;
     mark(ctx, VB_STAGE_DENSITY, 0);
-    recip_f32_kernel<<<(unsigned)((g->n + 255) / 256), 256, 0, s>>>(b, g->n, 1.f, ib);
-    density_const_kernel<<<(unsigned)((cl.B + 255) / 256), 256, 0, s>>>(eps2_dev, cl.B, cden);
-    switch (lpr) {
-        case 8: density_kernel<8><<<kRowBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, ib, cden, cl, psi); break;
-        case 16: density_kernel<16><<<kRowBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, ib, cden, cl, psi); break;
-        default: density_kernel<32><<<kRowBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, ib, cden, cl, psi); break;
+    if (aux.ib) {
+        ib = aux.ib;
+    } else {
+        recip_f32_kernel<<<(unsigned)((g->n + 255) / 256), 256, 0, s>>>(b, g->n, 1.f, ib);
+        ctx->launches += 1;
     }
-    density_finish_kernel<<<(unsigned)((g->n + 255) / 256), 256, 0, s>>>(b, eps2_dev, g->n, cl, d, beta, psi, P);
+    density_const_kernel<<<(unsigned)((cl.B + 255) / 256), 256, 0, s>>>(eps2_dev, cl.B, cden);
+    if (aux.t) {
+        density_kernel<8, true><<<kRowBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, ib, aux.t, cden, cl, psi);
+    } else {
+        switch (lpr) {
+            case 8: density_kernel<8, false><<<kRowBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, ib, nullptr, cden, cl, psi); break;
+            case 16: density_kernel<16, false><<<kRowBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, ib, nullptr, cden, cl, psi); break;
+            default: density_kernel<32, false><<<kRowBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, ib, nullptr, cden, cl, psi); break;
+        }
+    }
+    density_finish_kernel<<<(unsigned)((g->n + 255) / 256), 256, 0, s>>>(b, eps2_dev, g->n, cl, d, beta, psi, P,
+                                                                                   aux.iP, aux.pv);
     mark(ctx, VB_STAGE_DENSITY, 1);
-    ctx->launches += 4;
+    ctx->launches += 3;
     return last_launch();
 }
 
 // ------------------------------------------------------------------ operator-sweep centre
-// Segmented like the sweeps: slot bl + cloud holds the two sums of one cloud's rows.
-// 1 / b and 1 / P of every point as one 8-byte record, so that each entry's gather is one load.
-__global__ void recip_bp_kernel(const double* __restrict__ b, const double* __restrict__ P, int64_t n, float2* bp)
+// Segmented like the sweeps: slot bl + cloud holds the sum of one cloud's rows.
+// t_ij = ed2_ij (r_i r_j) of every entry, r = 1 / b or 1 / P, and the sum of t over the off-diagonal
+// entries of every segment (the centre's two sums; they only decide xi_c, which is rounded to a
+// quarter).  The diagonal's zero carries the sign bit, which tells the sweeps to leave it out.  Bound by
+// the gathers of r: nearly every r_j is a 32-byte sector from L2 and a line of its own in L1 (73M
+// entries at 1M torus points: 2.3 GB from L2 and 0.25 ms of one L1 line a cycle; measured 0.38 ms with the
+// store of t, 0.24 ms without it when the rows are taken in spatial order, which costs as much
+// again in scattered row reads and writes and is not done).  So a build gathers once per bandwidth, here, and the
+// passes over t only stream it.
+__global__ void __launch_bounds__(kRowThreads) pair_kernel(const int64_t* __restrict__ row_ptr,
+                                                         const int32_t* __restrict__ col,
+                                                         const float* __restrict__ ed2, int64_t n,
+                                                         const float* __restrict__ rr, Clouds cl, float* tt,
+                                                         double* partial)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) bp[i] = make_float2((float)(1.0 / b[i]), (float)(1.0 / P[i]));
-}
-
-__global__ void __launch_bounds__(kRowThreads) centre_kernel(const int64_t* __restrict__ row_ptr,
-                                                           const int32_t* __restrict__ col,
-                                                           const float* __restrict__ ed2, int64_t n,
-                                                           const float2* __restrict__ bp, Clouds cl, double* partial)
-{
-    __shared__ double sh[WARPS][2];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int LPR = 8, RPB = WARPS * 32 / LPR;   // lanes per row, rows per block and step
+    __shared__ double sh[WARPS];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane % LPR;
+    const bool vec = aligned16(col, ed2) && aligned16(tt, tt);
     const int64_t per = rows_per_block(n, gridDim.x);
     const int64_t r0 = min(n, (int64_t)blockIdx.x * per), r1 = min(n, r0 + per);
     if (r0 >= r1) return;
     const int cf = cloud_of(cl.ptr, cl.B, r0), cla = cloud_of(cl.ptr, cl.B, r1 - 1);
     for (int cb = cf; cb <= cla; ++cb) {
         const int64_t s0 = max(r0, cloud_lo(cl, cb)), s1 = min(r1, cloud_hi(cl, cb, n));
-        double a_op = 0.0, a_den = 0.0;
-        for (int64_t i = s0 + w; i < s1; i += WARPS) {
-            const int64_t rb = row_ptr[i], re = row_ptr[i + 1];
-            const float2 bpi = bp[i];
-            const float pi_ = bpi.y, bi = bpi.x;
-            float so = 0.f, sd = 0.f;
-            for (int64_t e0 = rb + lane; e0 < re; e0 += UNR * 32) {
+        double a = 0.0;
+        for (int64_t base = s0; base < s1; base += RPB) {
+            const int64_t r = base + threadIdx.x / LPR;
+            const bool ok = r < s1;
+            const int64_t rb = ok ? row_ptr[r] : 0, re = ok ? row_ptr[r + 1] : 0;
+            const float ri = ok ? rr[r] : 0.f;
+            float s = 0.f;
+            for (int64_t e0 = quad_start(rb, sub); e0 < re; e0 += 4 * LPR) {
                 int32_t jj[UNR];
-                float xx[UNR];
-                load_entries<32>(col, ed2, e0, re, jj, xx);
-                float2 bj[UNR];
+                float xx[UNR], tq[UNR];
+                load_quad(col, ed2, vec, e0, rb, re, jj, xx);
 #pragma unroll
-                for (int u = 0; u < UNR; ++u)
-                    if (jj[u] >= 0) bj[u] = bp[jj[u]];
+                for (int u = 0; u < UNR; ++u) tq[u] = jj[u] >= 0 ? rr[jj[u]] : 0.f;
 #pragma unroll
                 for (int u = 0; u < UNR; ++u) {
-                    const int32_t j = jj[u];
-                    if (j < 0 || j == i) continue;
-                    so += xx[u] * (pi_ * bj[u].y);
-                    sd += xx[u] * (bi * bj[u].x);
+                    tq[u] = xx[u] * (ri * tq[u]);
+                    if (jj[u] == r) tq[u] = -0.f;
+                    s += tq[u];
+                }
+                if (!tt) continue;
+                if (vec && e0 >= rb && e0 + 3 < re) {
+                    *(float4*)(tt + e0) = make_float4(tq[0], tq[1], tq[2], tq[3]);
+                } else {
+#pragma unroll
+                    for (int u = 0; u < UNR; ++u)
+                        if (jj[u] >= 0) tt[e0 + u] = tq[u];
                 }
             }
-            so = warp_sum_f32(so);   // FP32 tree over the lanes; the FP64 pipe is narrow
-            sd = warp_sum_f32(sd);
-            a_op += (double)so;
-            a_den += (double)sd;
+            a += (double)warp_sum_f32(s);   // FP32 tree over the warp's four rows; the FP64 pipe is narrow
         }
-        if (lane == 0) { sh[w][0] = a_op; sh[w][1] = a_den; }
+        if (lane == 0) sh[w] = a;
         __syncthreads();
-        if (threadIdx.x < 2) {
+        if (threadIdx.x == 0) {
             double sum = 0.0;
-            for (int ww = 0; ww < WARPS; ++ww) sum += sh[ww][threadIdx.x];
-            partial[2 * ((int64_t)blockIdx.x + cb) + threadIdx.x] = sum;
+            for (int ww = 0; ww < WARPS; ++ww) sum += sh[ww];
+            partial[(int64_t)blockIdx.x + cb] = sum;
         }
         __syncthreads();
     }
 }
 
-// One block per cloud.
-__global__ void __launch_bounds__(SEG_T) centre_finish_kernel(const double* __restrict__ partial, int nblk, int64_t n,
-                                                              Clouds cl, double* xi_c)
+// One block per cloud: the two sums over the cloud's slots, every thread a fixed share of them.
+constexpr int CEN_T = 256;
+__global__ void __launch_bounds__(CEN_T) centre_finish_kernel(const double* __restrict__ p_op,
+                                                            const double* __restrict__ p_den, int nblk, int64_t n,
+                                                            Clouds cl, double* xi_c)
 {
-    __shared__ double part[SEG_PARTS * SEG_COLS];
-    __shared__ double tot[2];
-    const int b = blockIdx.x;
-    seg_totals(partial, 2, cl, b, n, nblk, part, tot);
-    // R9: the operator argument is ed2 / (4 P_i P_j); tot[0] holds sum ed2 / (P_i P_j)
-    if (threadIdx.x == 0) xi_c[b] = floor(4.0 * log2(0.25 * tot[0] / tot[1]) + 0.5) / 4.0;
+    __shared__ double sh[CEN_T / 32][2];
+    const int b = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t per = rows_per_block(n, nblk);
+    const int64_t lo = cloud_lo(cl, b), hi = cloud_hi(cl, b, n);
+    double so = 0.0, sd = 0.0;
+    for (int64_t bl = lo / per + threadIdx.x; bl <= (hi - 1) / per; bl += CEN_T) {
+        so += p_op[bl + b];
+        sd += p_den[bl + b];
+    }
+    so = warp_sum_f64(so);
+    sd = warp_sum_f64(sd);
+    if (lane == 0) { sh[w][0] = so; sh[w][1] = sd; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        so = sd = 0.0;
+        for (int q = 0; q < CEN_T / 32; ++q) { so += sh[q][0]; sd += sh[q][1]; }
+        // R9: the operator argument is ed2 / (4 P_i P_j); so holds sum ed2 / (P_i P_j)
+        xi_c[b] = floor(4.0 * log2(0.25 * so / sd) + 0.5) / 4.0;
+    }
 }
 
 size_t centre_ws_bytes(int64_t n, int B)
 {
     Carve c(nullptr);
-    c.take<float2>(n);
+    c.take<float>(2 * n);
     c.take<double>(seg_slots(B) * 2);
     return c.off;
 }
+size_t pair_slots(int B) { return seg_slots(B); }
+
+vb_status pair_run(Ctx* ctx, const vb_graph* g, const float* r, float* t, double* partial, Clouds cl)
+{
+    pair_kernel<<<kRowBlocks, kRowThreads, 0, ctx->stream>>>(g->row_ptr, g->col, g->ed2, g->n, r, cl, t, partial);
+    ctx->launches += 1;
+    return last_launch();
+}
 
 vb_status centre_run(Ctx* ctx, const vb_graph* g, const double* b, const double* P, double* xi_c_dev, void* ws,
-                     size_t ws_bytes, Clouds cl)
+                     size_t ws_bytes, Clouds cl, const BuildAux& aux)
 {
     if (!g || !g->row_ptr || !b || !P || !xi_c_dev) return VB_ERR_ARG;
     if (cl.B < 1 || (cl.B > 1 && !cl.ptr)) return VB_ERR_ARG;
     Carve c(ws);
-    float2* bp = c.take<float2>(g->n);
+    float* rr = c.take<float>(2 * g->n);
     double* partial = c.take<double>(seg_slots(cl.B) * 2);
     if (!ws || ws_bytes < c.off) return VB_ERR_WORKSPACE;
     cudaStream_t s = ctx->stream;
+    const unsigned gn = (unsigned)((g->n + 255) / 256);
+    const double* p_den = aux.part_den;
     mark(ctx, VB_STAGE_CENTRE, 0);
-    recip_bp_kernel<<<(unsigned)((g->n + 255) / 256), 256, 0, s>>>(b, P, g->n, bp);
-    centre_kernel<<<kRowBlocks, kRowThreads, 0, s>>>(g->row_ptr, g->col, g->ed2, g->n, bp, cl, partial);
-    centre_finish_kernel<<<(unsigned)cl.B, SEG_T, 0, s>>>(partial, kRowBlocks, g->n, cl, xi_c_dev);
+    const float* iP = aux.iP;
+    if (!iP) {   // outside a build: both reciprocals, and the bandwidths' sum without its products
+        double* pd = partial + seg_slots(cl.B);
+        recip_f32_kernel<<<gn, 256, 0, s>>>(b, g->n, 1.f, rr);
+        recip_f32_kernel<<<gn, 256, 0, s>>>(P, g->n, 1.f, rr + g->n);
+        vb_status st = pair_run(ctx, g, rr, nullptr, pd, cl);
+        if (st != VB_OK) return st;
+        iP = rr + g->n;
+        p_den = pd;
+        ctx->launches += 2;
+    }
+    vb_status st = pair_run(ctx, g, iP, aux.t, partial, cl);
+    if (st != VB_OK) return st;
+    centre_finish_kernel<<<(unsigned)cl.B, CEN_T, 0, s>>>(partial, p_den, kRowBlocks, g->n, cl, xi_c_dev);
     mark(ctx, VB_STAGE_CENTRE, 1);
-    ctx->launches += 3;
+    ctx->launches += 1;
     return last_launch();
 }
 
 // ------------------------------------------------------------------ a12 / a13 operator and L-hat
-// The per-point values every entry gathers from its column j, packed in one 16-byte record so
-// that a gather is one sector: 1 / P as an unevaluated pair (hi, lo) of floats, q^-alpha (set
-// by the q pass) and 1 / S (set by the D pass).
-struct __align__(16) PointOp {
-    float iPh, iPl, qa, iS;
-};
-
 __global__ void recip_pair_kernel(const double* __restrict__ v, int64_t n, PointOp* pv)
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -865,7 +967,7 @@ size_t kernel_csr_ws_bytes(int64_t n, int B)
 
 vb_status kernel_csr_run(Ctx* ctx, const vb_graph* g, const double* psi, const double* P, const vb_op_params* op,
                          const double* eps2_op_dev, float* val, double* q, double* D, double* S, void* ws,
-                         size_t ws_bytes, Clouds cl, int lpr)
+                         size_t ws_bytes, Clouds cl, int lpr, const BuildAux& aux)
 {
     if (!g || !g->row_ptr || !psi || !P || !op || !eps2_op_dev || !val || !q || !D || !S) return VB_ERR_ARG;
     if (!(op->d > 0) || cl.B < 1 || (cl.B > 1 && !cl.ptr)) return VB_ERR_ARG;
@@ -878,7 +980,12 @@ vb_status kernel_csr_run(Ctx* ctx, const vb_graph* g, const double* psi, const d
     cudaStream_t s = ctx->stream;
     const int64_t n = g->n;
     mark(ctx, VB_STAGE_OPERATOR, 0);
-    recip_pair_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(P, n, pv);
+    if (aux.pv) {
+        pv = aux.pv;
+    } else {
+        recip_pair_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(P, n, pv);
+        ctx->launches += 1;
+    }
     op_const_kernel<<<(unsigned)((cl.B + 255) / 256), 256, 0, s>>>(eps2_op_dev, cl.B, cop);
 #define VB_ROWS(K, ...)                                                        \
     switch (lpr) {                                                             \
@@ -906,7 +1013,7 @@ vb_status kernel_csr_run(Ctx* ctx, const vb_graph* g, const double* psi, const d
 #undef VB_ROWS
 #undef VB_ROWS2
     mark(ctx, VB_STAGE_LHAT, 1);
-    ctx->launches += 3;
+    ctx->launches += 2;
     return last_launch();
 }
 

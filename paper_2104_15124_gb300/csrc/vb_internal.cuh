@@ -131,6 +131,24 @@ constexpr int kMaxGrid = 64;          // epsilon sweep grid points per launch
 constexpr int kRowBlocks = 152 * 8;   // fixed grid of the row passes (deterministic reductions)
 constexpr int kRowThreads = 256;
 
+// ------------------------------------------------------------------ per-point records of the row passes
+// The per-point values every entry gathers from its column j, packed in one 16-byte record so
+// that a gather is one sector: 1 / P as an unevaluated pair (hi, lo) of floats, q^-alpha (set
+// by the q pass) and 1 / S (set by the D pass).
+struct __align__(16) PointOp {
+    float iPh, iPl, qa, iS;
+};
+
+// What a build computes once and its passes share (all null outside a build: every pass then
+// prepares its own).
+struct BuildAux {
+    float* ib = nullptr;               // 1 / b
+    float* iP = nullptr;               // 1 / P
+    PointOp* pv = nullptr;             // 1 / P as a pair; q^-alpha and 1 / S as they are formed
+    float* t = nullptr;                // per entry: ed2 / (b_i b_j), later ed2 / (P_i P_j) (the room of L-hat's values)
+    double* part_den = nullptr;        // pair_slots sums of ed2 / (b_i b_j)
+};
+
 // ------------------------------------------------------------------ launch wrappers (defined per .cu)
 // kNN (knn.cu)
 size_t gradient_ws_bytes(int64_t n, int32_t ell, int32_t m);
@@ -156,23 +174,29 @@ vb_status order_run(Ctx* ctx, const float* x, int64_t n, int32_t m, void* ws, si
 size_t graph_plan_bytes(int64_t n, int32_t k);
 vb_status graph_run(Ctx* ctx, int64_t n, int32_t k, const int32_t* nbr, const double* nbr_d2, int64_t* row_ptr,
                     int32_t* col, float* ed2, int64_t cap, int64_t* nnz_dev, void* ws, size_t ws_bytes);
-vb_status bandwidth_run(Ctx* ctx, int64_t n, int32_t k, int32_t k_bw, const double* nbr_d2, double* b);
+vb_status bandwidth_run(Ctx* ctx, int64_t n, int32_t k, int32_t k_bw, const double* nbr_d2, double* b,
+                        float* ib = nullptr);
 // row passes (passes.cu)
 // Per-cloud scalars (eps^2, xi_c, chi, dimension) are arrays of cl.B entries (chi: cl.B x G).
 size_t sweep_ws_bytes(int64_t n, int B = 1);
 vb_status sweep_run(Ctx* ctx, const vb_graph* g, const double* rho, double scale, const double* xi_c_dev,
                     double xi_lo, double xi_hi, double dxi, int warn_bit, double* eps2, double* chi, double* dim,
-                    void* ws, size_t ws_bytes, Clouds cl = Clouds());
+                    void* ws, size_t ws_bytes, Clouds cl = Clouds(), const float* irho_ready = nullptr,
+                    const float* t_ready = nullptr);
 size_t density_ws_bytes(int64_t n, int B = 1);
 vb_status density_run(Ctx* ctx, const vb_graph* g, const double* b, const double* eps2_dev, double d, double beta,
-                      double* psi, double* P, void* ws, size_t ws_bytes, Clouds cl = Clouds(), int lpr = 8);
+                      double* psi, double* P, void* ws, size_t ws_bytes, Clouds cl = Clouds(), int lpr = 8,
+                      const BuildAux& aux = BuildAux());
 size_t centre_ws_bytes(int64_t n, int B = 1);
+// t = ed2 (r_i r_j) of every entry and its sums per segment (pair_slots(B) FP64)
+size_t pair_slots(int B);
+vb_status pair_run(Ctx* ctx, const vb_graph* g, const float* r, float* t, double* partial, Clouds cl);
 vb_status centre_run(Ctx* ctx, const vb_graph* g, const double* b, const double* P, double* xi_c_dev, void* ws,
-                     size_t ws_bytes, Clouds cl = Clouds());
+                     size_t ws_bytes, Clouds cl = Clouds(), const BuildAux& aux = BuildAux());
 size_t kernel_csr_ws_bytes(int64_t n, int B = 1);
 vb_status kernel_csr_run(Ctx* ctx, const vb_graph* g, const double* psi, const double* P, const vb_op_params* op,
                          const double* eps2_op_dev, float* val, double* q, double* D, double* S, void* ws,
-                         size_t ws_bytes, Clouds cl = Clouds(), int lpr = 8);
+                         size_t ws_bytes, Clouds cl = Clouds(), int lpr = 8, const BuildAux& aux = BuildAux());
 size_t spmv_ws_bytes(int64_t n);
 vb_status spmv_lap_launch(cudaStream_t s, const vb_graph* g, const float* val, const double* S, float alpha,
                           const float* x, float beta, float* y, double* z, float* sf);
