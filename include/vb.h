@@ -376,7 +376,7 @@ vb_status vb_spmv(vb_ctx* ctx, const vb_graph* g, const float* val, const double
  * computes what vb_spmv() computes in VB_SPMV_LAPLACIAN mode, on the given
  * stream (a cudaStream_t; NULL = legacy default stream) of the current device.
  *   - Scratch: one static device array inside libvb, sized for
- *     VB_NOALLOC_MAX_N rows at 12 bytes per row (about 12.6 MB); every GPU
+ *     VB_NOALLOC_MAX_N rows at 16 bytes per row (about 16.8 MB); every GPU
  *     that loads the library holds it until the process exits.
  *   - The first call on each device resolves the array's device address
  *     (cudaGetSymbolAddress, with that device current) and caches it; make

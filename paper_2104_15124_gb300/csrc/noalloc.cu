@@ -7,9 +7,9 @@
 // and embeddings that run under a fixed device-memory budget.  They still
 // pass their inputs and outputs; only the scratch moves into the library.
 //
-// The scratch (z = x / S in FP64 and S in FP32, 12 bytes per row) lives in
+// The scratch (z = x / S as a pair of floats and S, a 16-byte record per row) lives in
 // the file-scope array g_lap_scratch, sized for VB_NOALLOC_MAX_N rows; every
-// GPU that loads libvb holds it (about 12.6 MB) until the process exits.  Host
+// GPU that loads libvb holds it (about 16.8 MB) until the process exits.  Host
 // code cannot use the array's name as a device address, so the first call on
 // each device, with that device current, resolves it once with
 // cudaGetSymbolAddress and caches the result.
@@ -20,8 +20,7 @@
 namespace {
 
 constexpr int64_t kMaxN = VB_NOALLOC_MAX_N;
-constexpr size_t kZBytes = ((size_t)kMaxN * sizeof(double) + 255) & ~(size_t)255;
-constexpr size_t kScratchBytes = kZBytes + (size_t)kMaxN * sizeof(float);
+constexpr size_t kScratchBytes = (size_t)kMaxN * sizeof(float4);
 
 static __device__ __align__(256) unsigned char g_lap_scratch[kScratchBytes];
 
@@ -54,7 +53,5 @@ extern "C" vb_status vb_spmv_laplacian_noalloc(void* stream, const vb_graph* g, 
     void* base = nullptr;
     vb_status st = scratch_address(&base);
     if (st != VB_OK) return st;
-    double* z = (double*)base;
-    float* sf = (float*)((char*)base + kZBytes);
-    return vb::spmv_lap_launch((cudaStream_t)stream, g, val, S, alpha, x, beta, y, z, sf);
+    return vb::spmv_lap_launch((cudaStream_t)stream, g, val, S, alpha, x, beta, y, (float4*)base);
 }

@@ -34,3 +34,32 @@ def test_build_equals_its_steps(n, m, k, c):
     for r in range(k):
         ref = ref + out.nbr_d2[:, r].cpu().numpy()
     assert np.array_equal(b.cpu().numpy(), np.sqrt(ref))
+
+
+@pytest.mark.parametrize("offset", [0, 1, 3])
+def test_difference_form_product_at_any_alignment(offset):
+    # rows of one to many entries, arrays that do and do not start on 16 bytes, and an infinite input:
+    # FP64 sums of the same FP32 entries within the rounding of FP32 sums of 2 k + 1 terms
+    import paper_2104_15124_gb300 as vb
+    r = np.random.default_rng(offset)
+    n = 1003
+    x = torch.from_numpy(r.standard_normal((n, 3)).astype(np.float32)).cuda()
+    out = vb.build(x, 20, d=2.0, c=1.0)
+    z = out.graph.nnz
+    col = torch.empty(z + 4, dtype=torch.int32, device="cuda")[offset:offset + z].copy_(out.graph.col[:z])
+    val = torch.empty(z + 4, dtype=torch.float32, device="cuda")[offset:offset + z].copy_(out.val[:z])
+    g = vb.Graph(n, out.graph.row_ptr, col, out.graph.ed2, out.graph.nnz_dev)
+    v = torch.from_numpy(r.standard_normal(n).astype(np.float32)).cuda()
+    row = torch.repeat_interleave(torch.arange(n, device="cuda"), g.row_ptr[1:] - g.row_ptr[:-1])
+    j = col.long()
+    zz = v.double() / out.S
+    t = val.double() * out.S[j] * (zz[j] - zz[row])
+    ref = torch.zeros(n, dtype=torch.float64, device="cuda").index_add_(0, row, t)
+    mag = torch.zeros(n, dtype=torch.float64, device="cuda").index_add_(0, row, t.abs())
+    y = vb.spmv(g, val, v, S=out.S, laplacian=True)
+    assert bool(((y.double() - ref).abs() <= 8 * 2.0 ** -24 * mag + 1e-30).all())
+    v[5] = float("inf")
+    y = vb.spmv(g, val, v, S=out.S, laplacian=True)
+    touched = torch.zeros(n, dtype=torch.bool, device="cuda")
+    touched[row[j == 5]] = True
+    assert not bool(y[~touched].isinf().any()) and bool(y[touched].isinf().all())
