@@ -247,12 +247,42 @@ __global__ void project_kernel(const float* __restrict__ Z, const float* __restr
 }
 
 // ------------------------------------------------------------------ host: small dense FP64 algebra
-// Cyclic Jacobi eigen-decomposition of a symmetric B x B matrix (row-major):
-// on return A's diagonal holds the eigenvalues and V the eigenvectors (columns).
-static void jacobi_eig(std::vector<double>& A, std::vector<double>& V, int B)
+// C (ra x cb) = A (ra x n) B (n x cb), rows of B taken in turn: every element is summed over k in
+// increasing order, as a dot product would, but along contiguous rows (a dot product down B's columns
+// cost a cache line per term).
+static void small_matmul(const double* A, const double* Bm, double* C, int ra, int n, int cb)
 {
-    V.assign((size_t)B * B, 0.0);
-    for (int i = 0; i < B; ++i) V[(size_t)i * B + i] = 1.0;
+    std::fill(C, C + (size_t)ra * cb, 0.0);
+    for (int i = 0; i < ra; ++i)
+        for (int k = 0; k < n; ++k) {
+            const double a = A[(size_t)i * n + k];
+            const double* br = Bm + (size_t)k * cb;
+            double* cr = C + (size_t)i * cb;
+            for (int j = 0; j < cb; ++j) cr[j] += a * br[j];
+        }
+}
+
+// (x, y) <- (c x - s y, s x + c y) along two rows, the second product of the difference fused, or the first.
+template <bool FUSE_SECOND>
+static void rotate_rows(double* __restrict__ x, double* __restrict__ y, int B, double c, double s)
+{
+    for (int k = 0; k < B; ++k) {
+        const double u = x[k], v = y[k];
+        x[k] = FUSE_SECOND ? std::fma(-s, v, c * u) : std::fma(c, u, -(s * v));
+        y[k] = std::fma(s, u, c * v);
+    }
+}
+
+// Cyclic Jacobi eigen-decomposition of a symmetric B x B matrix (row-major): on return A's diagonal
+// holds the eigenvalues and the rows of Vt the eigenvectors, which a rotation then updates along
+// memory (with the eigenvectors in columns a decomposition of order 96 took 5.7 ms of a Grace core, now
+// 3.8; two of them are most of a solver iteration's host time).  The fused operations are spelled out
+// because the filtered block's Gram matrix is singular to working precision: a last-bit difference here moves
+// the unconverged end of the block, and with it the last digits of every output.
+static void jacobi_eig(std::vector<double>& A, std::vector<double>& Vt, int B)
+{
+    Vt.assign((size_t)B * B, 0.0);
+    for (int i = 0; i < B; ++i) Vt[(size_t)i * B + i] = 1.0;
     for (int sweep = 0; sweep < 60; ++sweep) {
         double off = 0.0, tot = 0.0;
         for (int p = 0; p < B; ++p)
@@ -264,27 +294,21 @@ static void jacobi_eig(std::vector<double>& A, std::vector<double>& V, int B)
         if (off <= 1e-30 * tot || off == 0.0) break;
         for (int p = 0; p < B - 1; ++p)
             for (int q = p + 1; q < B; ++q) {
-                const double apq = A[(size_t)p * B + q];
+                double *rp = &A[(size_t)p * B], *rq = &A[(size_t)q * B];
+                const double apq = rp[q];
                 if (apq == 0.0) continue;
-                const double app = A[(size_t)p * B + p], aqq = A[(size_t)q * B + q];
+                const double app = rp[p], aqq = rq[q];
                 const double theta = (aqq - app) / (2.0 * apq);
                 const double tt = (theta >= 0 ? 1.0 : -1.0) / (std::fabs(theta) + std::sqrt(theta * theta + 1.0));
                 const double c = 1.0 / std::sqrt(tt * tt + 1.0), s = tt * c;
+                double *cp = &A[p], *cq = &A[q];
                 for (int k = 0; k < B; ++k) {   // columns p, q
-                    const double akp = A[(size_t)k * B + p], akq = A[(size_t)k * B + q];
-                    A[(size_t)k * B + p] = c * akp - s * akq;
-                    A[(size_t)k * B + q] = s * akp + c * akq;
+                    const double x = cp[(size_t)k * B], y = cq[(size_t)k * B];
+                    cp[(size_t)k * B] = std::fma(c, x, -(s * y));
+                    cq[(size_t)k * B] = std::fma(s, x, c * y);
                 }
-                for (int k = 0; k < B; ++k) {   // rows p, q
-                    const double apk = A[(size_t)p * B + k], aqk = A[(size_t)q * B + k];
-                    A[(size_t)p * B + k] = c * apk - s * aqk;
-                    A[(size_t)q * B + k] = s * apk + c * aqk;
-                }
-                for (int k = 0; k < B; ++k) {
-                    const double vkp = V[(size_t)k * B + p], vkq = V[(size_t)k * B + q];
-                    V[(size_t)k * B + p] = c * vkp - s * vkq;
-                    V[(size_t)k * B + q] = s * vkp + c * vkq;
-                }
+                rotate_rows<true>(rp, rq, B, c, s);
+                rotate_rows<false>(&Vt[(size_t)p * B], &Vt[(size_t)q * B], B, c, s);
             }
     }
 }
@@ -404,6 +428,7 @@ vb_status solve_run(Ctx* ctx, const vb_graph* g, int64_t cap, const float* val, 
 
     std::vector<double> theta(B, 0.0), prev(nwant, 0.0);
     std::vector<float> Mh((size_t)B * B);
+    std::vector<double> V1, V2, C1, C1t, T1, Hp, U, R;
     float* bufs[3] = {w.Z, w.Y, w.X};
     int zi = 0;   // which of bufs holds the current Ritz block
     double mu_cut = 0.5 * mu_max;
@@ -448,7 +473,6 @@ vb_status solve_run(Ctx* ctx, const vb_graph* g, int64_t cap, const float* val, 
                 Gh[(size_t)a * B + b] = Gh[(size_t)b * B + a] = gs;
             }
         // G = V diag(g) V^T; keep the r directions with g > 1e-12 max(g): C1 = V_r g_r^-1/2 (B x r)
-        std::vector<double> V1, V2;
         jacobi_eig(Gh, V1, B);
         double gmax = 0.0;
         for (int a = 0; a < B; ++a) gmax = std::max(gmax, Gh[(size_t)a * B + a]);
@@ -457,37 +481,34 @@ vb_status solve_run(Ctx* ctx, const vb_graph* g, int64_t cap, const float* val, 
             if (Gh[(size_t)a * B + a] > 1e-12 * gmax) keep.push_back(a);
         const int r = (int)keep.size();
         if (r < nwant) return VB_ERR_NOT_CONVERGED;
-        std::vector<double> C1((size_t)B * r);
+        C1.resize((size_t)B * r);
+        C1t.resize((size_t)r * B);
         for (int q = 0; q < r; ++q) {
             const double sc = 1.0 / std::sqrt(Gh[(size_t)keep[q] * B + keep[q]]);
-            for (int row = 0; row < B; ++row) C1[(size_t)row * r + q] = V1[(size_t)row * B + keep[q]] * sc;
+            for (int row = 0; row < B; ++row) {
+                const double v = V1[(size_t)keep[q] * B + row] * sc;
+                C1[(size_t)row * r + q] = v;
+                C1t[(size_t)q * B + row] = v;
+            }
         }
         // H' = C1^T H C1 (r x r), eigen-decomposed; Ritz vectors Y C1 U, values descending
-        std::vector<double> T1((size_t)B * r), Hp((size_t)r * r);
-        for (int row = 0; row < B; ++row)
-            for (int b = 0; b < r; ++b) {
-                double sacc = 0.0;
-                for (int k = 0; k < B; ++k) sacc += Hh[(size_t)row * B + k] * C1[(size_t)k * r + b];
-                T1[(size_t)row * r + b] = sacc;
-            }
-        for (int a = 0; a < r; ++a)
-            for (int b = 0; b < r; ++b) {
-                double sacc = 0.0;
-                for (int k = 0; k < B; ++k) sacc += C1[(size_t)k * r + a] * T1[(size_t)k * r + b];
-                Hp[(size_t)a * r + b] = sacc;
-            }
+        T1.resize((size_t)B * r);
+        Hp.resize((size_t)r * r);
+        small_matmul(Hh.data(), C1.data(), T1.data(), B, B, r);
+        small_matmul(C1t.data(), T1.data(), Hp.data(), r, B, r);
         jacobi_eig(Hp, V2, r);
         std::vector<int> ord(r);
         for (int a = 0; a < r; ++a) ord[a] = a;
         std::sort(ord.begin(), ord.end(), [&](int x, int y) { return Hp[(size_t)x * r + x] > Hp[(size_t)y * r + y]; });
         for (int a = 0; a < r; ++a) theta[a] = Hp[(size_t)ord[a] * r + ord[a]];
+        U.resize((size_t)r * r);
+        R.resize((size_t)B * r);
+        for (int k = 0; k < r; ++k)
+            for (int b = 0; b < r; ++b) U[(size_t)k * r + b] = V2[(size_t)ord[b] * r + k];
+        small_matmul(C1.data(), U.data(), R.data(), B, r, r);
         std::fill(Mh.begin(), Mh.end(), 0.f);
         for (int row = 0; row < B; ++row)
-            for (int b = 0; b < r; ++b) {
-                double sacc = 0.0;
-                for (int k = 0; k < r; ++k) sacc += C1[(size_t)row * r + k] * V2[(size_t)k * r + ord[b]];
-                Mh[(size_t)row * B + b] = (float)sacc;
-            }
+            for (int b = 0; b < r; ++b) Mh[(size_t)row * B + b] = (float)R[(size_t)row * r + b];
         if (cudaMemcpyAsync(w.M, Mh.data(), sizeof(float) * B * B, cudaMemcpyHostToDevice, s) != cudaSuccess)
             return VB_ERR_CUDA;
         // the rotated block goes to a buffer other than Yb
