@@ -107,7 +107,7 @@ size_t knn_plan(Carve& c, int64_t n, int32_t m, const vb_knn_params* p, KnnWs* w
     t.key[1] = c.take<uint32_t>(n);
     t.val[0] = c.take<uint32_t>(n);
     t.val[1] = c.take<uint32_t>(n);
-    t.hist = c.take<uint32_t>(256 * nblk);
+    t.hist = c.take<uint32_t>(256 * std::max<int64_t>(nblk, 128));
     t.hsum = c.take<uint32_t>((256 * nblk + USCAN_CHUNK - 1) / USCAN_CHUNK + 1);
     t.xs = c.take<float>(npad * mp);
     t.xs64 = c.take<double>(npad * mp);
@@ -159,37 +159,43 @@ __global__ void bbox_init_kernel(int* bbox, int* fb_count)
     if (t < 8) fb_count[t] = 0;
 }
 
-// Bounding box of the Morton coordinates; also rejects non-finite input.
-__global__ void bbox_kernel(const float* __restrict__ x, int64_t n, int m, int md, int* bbox, DevReport* rep)
+// Bounding box of the MD key coordinates (the first MD of rows of ld floats); also rejects
+// non-finite input.
+template <int MD>
+__global__ void bbox_kernel(const float* __restrict__ x, int64_t n, int ld, int* bbox, DevReport* rep)
 {
-    int lo[8], hi[8];
+    int lo[MD], hi[MD];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) { lo[r] = 0x7fffffff; hi[r] = (int)0x80000000; }
+    for (int r = 0; r < MD; ++r) { lo[r] = 0x7fffffff; hi[r] = (int)0x80000000; }
     bool bad = false;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        for (int r = 0; r < m; ++r) {
-            float v = x[i * m + r];
-            if (!isfinite(v)) bad = true;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                if (q == r && r < md) {
-                    int o = f2ord(v);
-                    lo[q] = min(lo[q], o);
-                    hi[q] = max(hi[q], o);
-                }
-            }
+        for (int r = 0; r < MD; ++r) {
+            const float v = x[i * ld + r];
+            bad |= !isfinite(v);
+            const int o = f2ord(v);
+            lo[r] = min(lo[r], o);
+            hi[r] = max(hi[r], o);
         }
     }
     if (bad) report_error(rep, VB_ERR_DEGENERATE);
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        int a = __reduce_min_sync(0xffffffffu, lo[r]);
-        int b = __reduce_max_sync(0xffffffffu, hi[r]);
-        if ((threadIdx.x & 31) == 0 && r < md) {
-            atomicMin(&bbox[r], a);
-            atomicMax(&bbox[8 + r], b);
+    for (int r = 0; r < MD; ++r) {
+        const int l = __reduce_min_sync(0xffffffffu, lo[r]), h = __reduce_max_sync(0xffffffffu, hi[r]);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMin(&bbox[r], l);
+            atomicMax(&bbox[8 + r], h);
         }
     }
+}
+
+// Rejects non-finite input among `count` values.
+__global__ void finite_kernel(const float* __restrict__ x, int64_t count, DevReport* rep)
+{
+    bool bad = false;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
+        bad |= !isfinite(x[i]);
+    if (bad) report_error(rep, VB_ERR_DEGENERATE);
 }
 
 // Hilbert curve index of md coordinates of `bits` bits each, by Skilling's transpose method
@@ -198,12 +204,14 @@ __global__ void bbox_kernel(const float* __restrict__ x, int64_t n, int m, int m
 // or exchange them with those of coordinate i), Gray-encode across the coordinates, then
 // interleave the bits as a Morton key would.  Consecutive indices are unit steps in space, so
 // the 64-point tiles of the order never straddle a jump of the curve, as Morton tiles can.
-__device__ __forceinline__ uint32_t hilbert_key(uint32_t (&X)[8], int md, int bits)
+template <int MD>
+__device__ __forceinline__ uint32_t hilbert_key(uint32_t (&X)[MD], int bits)
 {
     const uint32_t M = 1u << (bits - 1);
     for (uint32_t Q = M; Q > 1; Q >>= 1) {
         const uint32_t P = Q - 1;
-        for (int i = 0; i < md; ++i) {
+#pragma unroll
+        for (int i = 0; i < MD; ++i) {
             if (X[i] & Q) {
                 X[0] ^= P;
             } else {
@@ -213,51 +221,164 @@ __device__ __forceinline__ uint32_t hilbert_key(uint32_t (&X)[8], int md, int bi
             }
         }
     }
-    for (int i = 1; i < md; ++i) X[i] ^= X[i - 1];
+    for (int i = 1; i < MD; ++i) X[i] ^= X[i - 1];
     uint32_t t = 0;
     for (uint32_t Q = M; Q > 1; Q >>= 1)
-        if (X[md - 1] & Q) t ^= Q - 1;
-    for (int i = 0; i < md; ++i) X[i] ^= t;
+        if (X[MD - 1] & Q) t ^= Q - 1;
+    for (int i = 0; i < MD; ++i) X[i] ^= t;
     uint32_t k = 0;
     for (int b = bits - 1; b >= 0; --b)
-        for (int r = 0; r < md; ++r) k = (k << 1) | ((X[r] >> b) & 1u);
+        for (int r = 0; r < MD; ++r) k = (k << 1) | ((X[r] >> b) & 1u);
     return k;
 }
 
-__global__ void morton_kernel(const float* __restrict__ x, int64_t n, int m, int md, int bits,
-                              const int* __restrict__ bbox, uint32_t* key, uint32_t* val, int hilbert)
+// Sort key of a point: its MD key coordinates quantised to `bits` bits each within the bounding box,
+// then the Hilbert index or the Morton interleave of them.
+template <int MD>
+__device__ __forceinline__ uint32_t order_key(const float* __restrict__ row, int bits, const int* __restrict__ bbox,
+                                              bool hilbert)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
     const float qmax = (float)((1u << bits) - 1u);
-    uint32_t q[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int r = 0; r < md; ++r) {
-        float lo = ord2f(bbox[r]), hi = ord2f(bbox[8 + r]);
-        float ext = hi - lo;
-        float s = ext > 0.f ? qmax / ext : 0.f;
-        float v = fminf(fmaxf((x[i * m + r] - lo) * s, 0.f), qmax);
+    uint32_t q[MD];
+#pragma unroll
+    for (int r = 0; r < MD; ++r) {
+        const float lo = ord2f(bbox[r]), hi = ord2f(bbox[8 + r]);
+        const float ext = hi - lo;
+        const float s = ext > 0.f ? qmax / ext : 0.f;
+        const float v = fminf(fmaxf((row[r] - lo) * s, 0.f), qmax);
         q[r] = min((uint32_t)v, (1u << bits) - 1u);
     }
+    if (hilbert) return hilbert_key<MD>(q, bits);
     uint32_t k = 0;
-    if (hilbert) {
-        k = hilbert_key(q, md, bits);
-    } else {
-        for (int b = bits - 1; b >= 0; --b)
-            for (int r = 0; r < md; ++r) k = (k << 1) | ((q[r] >> b) & 1u);
-    }
-    key[i] = k;
+    for (int b = bits - 1; b >= 0; --b)
+#pragma unroll
+        for (int r = 0; r < MD; ++r) k = (k << 1) | ((q[r] >> b) & 1u);
+    return k;
+}
+
+template <int MD>
+__global__ void morton_kernel(const float* __restrict__ x, int64_t n, int ld, int bits, const int* __restrict__ bbox,
+                              uint32_t* key, uint32_t* val, int hilbert)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    key[i] = order_key<MD>(x + i * ld, bits, bbox, hilbert);
     val[i] = (uint32_t)i;
+}
+
+// The whole order of a cloud of at most SMALL_N points in one block: bounding box, keys, a bitonic
+// sort of (key, index) in shared memory (the order a stable radix sort gives), the sorted
+// coordinates, tile and super-tile boxes.  The separate passes are 19 launches of a few
+// microseconds each: 105 -> 29 us for 2,000 points.  The key coordinates are the first MD of the rows
+// kx (the input itself, or the projections on the principal axes).
+constexpr int SMALL_N = 4096, SMALL_T = 1024;
+template <int MD>
+__global__ void __launch_bounds__(SMALL_T) small_order_kernel(const float* __restrict__ x, const float* __restrict__ kx,
+                                                            int kld, int n, int npad, int m, int mp, int bits,
+                                                            int hilbert, uint32_t* perm, float* xs, double* xs64,
+                                                            float* tlo, float* thi, float* slo, float* shi,
+                                                            int* fb_count, DevReport* rep)
+{
+    __shared__ uint64_t key[SMALL_N];
+    __shared__ int bbox[16];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    if (t < 8) { bbox[t] = 0x7fffffff; fb_count[t] = 0; }
+    else if (t < 16) bbox[t] = (int)0x80000000;
+    __syncthreads();
+    int lo[MD], hi[MD];
+#pragma unroll
+    for (int r = 0; r < MD; ++r) { lo[r] = 0x7fffffff; hi[r] = (int)0x80000000; }
+    bool bad = false;
+    for (int i = t; i < n; i += SMALL_T) {
+#pragma unroll
+        for (int r = 0; r < MD; ++r) {
+            const float v = kx[(int64_t)i * kld + r];
+            bad |= !isfinite(v);
+            const int o = f2ord(v);
+            lo[r] = min(lo[r], o);
+            hi[r] = max(hi[r], o);
+        }
+    }
+    if (bad) report_error(rep, VB_ERR_DEGENERATE);
+#pragma unroll
+    for (int r = 0; r < MD; ++r) {
+        const int l = __reduce_min_sync(0xffffffffu, lo[r]), h = __reduce_max_sync(0xffffffffu, hi[r]);
+        if (lane == 0) {
+            atomicMin(&bbox[r], l);
+            atomicMax(&bbox[8 + r], h);
+        }
+    }
+    __syncthreads();
+    int P = 64;
+    while (P < n) P <<= 1;
+    for (int i = t; i < P; i += SMALL_T)
+        key[i] = i < n ? ((uint64_t)order_key<MD>(kx + (int64_t)i * kld, bits, bbox, hilbert) << 32) | (uint32_t)i : ~0ull;
+    __syncthreads();
+    for (int size = 2; size <= P; size <<= 1) {
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int i = t; i < P / 2; i += SMALL_T) {
+                const int a = 2 * i - (i & (stride - 1)), b = a + stride;
+                const uint64_t u = key[a], v = key[b];
+                if ((u > v) == ((a & size) == 0)) { key[a] = v; key[b] = u; }
+            }
+            // strides below 32 stay within a warp's 64 consecutive keys
+            if (stride > 32) __syncthreads();
+            else __syncwarp();
+            if (stride == 1 && size >= 64) __syncthreads();
+        }
+    }
+    __syncthreads();
+    for (int i = t; i < n; i += SMALL_T) perm[i] = (uint32_t)key[i];
+    for (int e = t; e < npad * mp; e += SMALL_T) {
+        const int p = e / mp, r = e - p * mp;
+        const float v = p < n && r < m ? x[(int64_t)(uint32_t)key[p] * m + r] : 0.f;
+        xs[e] = v;
+        xs64[e] = (double)v;
+    }
+    __syncthreads();   // the block's own writes of xs
+    const int ntiles = (n + TILE - 1) / TILE;
+    for (int tile = w; tile < ntiles; tile += SMALL_T / 32) {
+        const int p0 = tile * TILE + lane, p1 = p0 + 32;
+        for (int r = 0; r < mp; ++r) {
+            float l = INFINITY, h = -INFINITY;
+            if (p0 < n) { l = xs[p0 * mp + r]; h = l; }
+            if (p1 < n) { const float v = xs[p1 * mp + r]; l = fminf(l, v); h = fmaxf(h, v); }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                l = fminf(l, __shfl_xor_sync(0xffffffffu, l, o));
+                h = fmaxf(h, __shfl_xor_sync(0xffffffffu, h, o));
+            }
+            if (lane == 0) {
+                tlo[tile * mp + r] = r < m ? l : 0.f;
+                thi[tile * mp + r] = r < m ? h : 0.f;
+            }
+        }
+    }
+    __syncthreads();
+    for (int r = w; r < mp; r += SMALL_T / 32) {   // one super-tile at most
+        float l = lane < ntiles ? tlo[lane * mp + r] : INFINITY, h = lane < ntiles ? thi[lane * mp + r] : -INFINITY;
+        if (lane + 32 < ntiles) {
+            l = fminf(l, tlo[(lane + 32) * mp + r]);
+            h = fmaxf(h, thi[(lane + 32) * mp + r]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            l = fminf(l, __shfl_xor_sync(0xffffffffu, l, o));
+            h = fmaxf(h, __shfl_xor_sync(0xffffffffu, h, o));
+        }
+        if (lane == 0) { slo[r] = l; shi[r] = h; }
+    }
 }
 
 // ---- m > 4: the Morton key is built on the projections onto the cloud's PCA_D leading
 // principal axes, so that 64-point tiles are compact in the directions the points spread
 // along (the first coordinates of a wide input need not be those).  The axes only decide
 // the order of the search; the neighbour lists are exact whatever they are.
-constexpr int PCA_SAMPLE = 16384;   // rows sampled for the second moments
-constexpr int PCA_ROWS = 64;        // sampled rows staged per step
-constexpr int PCA_BLOCKS = 16;      // blocks of the moment pass (few, so few atomics)
-constexpr int PCA_EPT = 65;         // moments per thread: (128 * 128 + 128) / 256 rounded up
-constexpr int PCA_ITERS = 40;       // subspace iterations
+constexpr int PCA_SAMPLE = 8192;    // rows sampled for the second moments
+constexpr int PCA_ROWS = 32;        // sampled rows staged per step
+constexpr int PCA_BLOCKS = 152;     // blocks of the moment pass
+constexpr int PCA_EPT = 33;         // moments per thread: (128 * 129 / 2 + 128) / 256 rounded up
+constexpr int PCA_ITERS = 16;       // subspace iterations (on C^2)
 
 __global__ void pca_zero_kernel(double* mom, int64_t len)
 {
@@ -265,100 +386,130 @@ __global__ void pca_zero_kernel(double* mom, int64_t len)
         mom[i] = 0.0;
 }
 
-// Sampled first and second moments: mom[0] = rows, mom[1 + r] = sum x_r, mom[1 + m + r m + c] = sum x_r x_c.
-// Each of PCA_BLOCKS blocks sums its share of the sampled rows in FP32 registers, then adds
-// them to the FP64 totals once.
+// Sampled first and second moments: mom[0] = rows, mom[1 + r] = sum x_r, mom[1 + m + r m + c] = sum x_r x_c
+// for r <= c.  Each of PCA_BLOCKS blocks sums its share of the sampled rows in FP32 registers, then
+// adds them to the FP64 totals once.  (16 blocks summing all m^2 moments, with a division per moment and
+// row chunk: 966 us at m = 100, 222 us at m = 8.)
 __global__ void __launch_bounds__(256) pca_moments_kernel(const float* __restrict__ x, int64_t n, int m, int64_t stride,
                                                         int64_t rows, double* mom)
 {
-    __shared__ float xs[PCA_ROWS][128];
+    __shared__ float xs[PCA_ROWS][129];   // column m: ones, so that the first moments are products too
     const int t = threadIdx.x;
-    const int ne = m * m + m;
+    const int ne = (m + 1) * (m + 2) / 2 - 1;   // pairs a <= b of 0 .. m but (m, m)
     float acc[PCA_EPT];
+    int ab[PCA_EPT];
 #pragma unroll
-    for (int j = 0; j < PCA_EPT; ++j) acc[j] = 0.f;
+    for (int j = 0; j < PCA_EPT; ++j) {
+        acc[j] = 0.f;
+        int e = t + j * 256, a = 0;
+        if (e < ne) {   // e counts the pairs row by row: row a has m + 1 - a of them
+            a = (int)((2.f * (m + 1) + 1.f - sqrtf((2.f * (m + 1) + 1.f) * (2.f * (m + 1) + 1.f) - 8.f * e)) * 0.5f);
+            while (a > 0 && a * (m + 1) - a * (a - 1) / 2 > e) --a;
+            while ((a + 1) * (m + 1) - (a + 1) * a / 2 <= e) ++a;
+            ab[j] = a << 8 | (e - (a * (m + 1) - a * (a - 1) / 2) + a);
+        } else {
+            ab[j] = m << 8 | m;
+        }
+    }
+    const int nj = (ne + 255) / 256;
     int64_t taken = 0;
     for (int64_t r0 = (int64_t)blockIdx.x * PCA_ROWS; r0 < rows; r0 += (int64_t)gridDim.x * PCA_ROWS) {
         const int nr = (int)min((int64_t)PCA_ROWS, rows - r0);
         __syncthreads();
-        for (int i = t; i < nr * m; i += blockDim.x) {
-            const int rr = i / m, c = i - rr * m;
-            xs[rr][c] = x[(r0 + rr) * stride * m + c];
+        for (int i = t; i < PCA_ROWS * (m + 1); i += blockDim.x) {
+            const int rr = i / (m + 1), c = i - rr * (m + 1);
+            xs[rr][c] = rr >= nr ? 0.f : c == m ? 1.f : x[(r0 + rr) * stride * m + c];
         }
         __syncthreads();
         taken += nr;
 #pragma unroll
         for (int j = 0; j < PCA_EPT; ++j) {
-            const int e = t + j * 256;
-            if (e < m * m) {
-                const int a = e / m, b = e - a * m;
-                for (int rr = 0; rr < nr; ++rr) acc[j] = fmaf(xs[rr][a], xs[rr][b], acc[j]);
-            } else if (e < ne) {
-                const int a = e - m * m;
-                for (int rr = 0; rr < nr; ++rr) acc[j] += xs[rr][a];
-            }
+            if (j >= nj) break;
+            const int a = ab[j] >> 8, b = ab[j] & 255;
+#pragma unroll 8
+            for (int rr = 0; rr < PCA_ROWS; ++rr) acc[j] = fmaf(xs[rr][a], xs[rr][b], acc[j]);
         }
     }
 #pragma unroll
     for (int j = 0; j < PCA_EPT; ++j) {
-        const int e = t + j * 256;
-        if (e < m * m) atomicAdd(&mom[1 + m + e], (double)acc[j]);
-        else if (e < ne) atomicAdd(&mom[1 + (e - m * m)], (double)acc[j]);
+        const int a = ab[j] >> 8, b = ab[j] & 255;
+        if (t + j * 256 >= ne || taken == 0) continue;
+        atomicAdd(b == m ? &mom[1 + a] : &mom[1 + m + a * m + b], (double)acc[j]);
     }
-    if (t == 0) atomicAdd(&mom[0], (double)taken);
+    if (t == 0 && taken) atomicAdd(&mom[0], (double)taken);
 }
 
-// One block: covariance from the moments, then PCA_ITERS steps of subspace iteration
-// V <- orth(C V) for PCA_D columns (modified Gram-Schmidt); writes V (m x PCA_D).
+// One block: covariance from the moments, its square (a subspace step with it counts for two), then
+// PCA_ITERS steps V <- orth(C^2 V) for PCA_D columns, C^2 in shared memory and the orthogonalisation
+// (modified Gram-Schmidt) inside one warp; writes V (m x PCA_D).  40 steps on C from global memory with
+// three block barriers per inner product took 385 us at m = 100.
 __global__ void __launch_bounds__(256) pca_axes_kernel(double* mom, int m, float* C)
 {
-    __shared__ float V[128][PCA_D], Wm[128][PCA_D];
-    __shared__ float red[8];
+    extern __shared__ float C2[];   // [m][m + 1]
+    __shared__ float V[PCA_D][128], Wm[PCA_D][128];
+    __shared__ float s_inv;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const double N = fmax(mom[0], 1.0);
     const double* mu = mom + 1;
     const double* S = mom + 1 + m;
     for (int i = t; i < m * m; i += blockDim.x) {   // covariance, FP32 from here on
         const int r = i / m, c = i - r * m;
-        C[i] = (float)(S[i] / N - (mu[r] / N) * (mu[c] / N));
+        C[i] = (float)(S[min(r, c) * m + max(r, c)] / N - (mu[r] / N) * (mu[c] / N));
     }
     for (int i = t; i < m * PCA_D; i += blockDim.x) {   // a fixed, well-spread start
         const int r = i / PCA_D, d = i - r * PCA_D;
         const uint32_t h = (uint32_t)(r * 2654435761u) ^ (uint32_t)(d * 40503u + 0x9e3779b9u);
-        V[r][d] = (float)((h >> 8) & 0xffff) / 65536.f - 0.5f + (r % PCA_D == d ? 1.f : 0.f);
+        V[d][r] = (float)((h >> 8) & 0xffff) / 65536.f - 0.5f + (r % PCA_D == d ? 1.f : 0.f);
+    }
+    __syncthreads();
+    if (w == 0) {   // scale: the trace, so that the square stays in range
+        float tr = 0.f;
+        for (int r = lane; r < m; r += 32) tr += C[r * m + r];
+        tr = warp_sum_f32(tr);
+        if (lane == 0) s_inv = tr > 0.f && isfinite(tr) ? 1.f / tr : 0.f;
+    }
+    __syncthreads();
+    const float inv = s_inv;
+    for (int i = t; i < m * m; i += blockDim.x) {
+        const int r = i / m, c = i - r * m;
+        float acc = 0.f;
+        for (int k = 0; k < m; ++k) acc = fmaf(C[k * m + r] * inv, C[k * m + c] * inv, acc);   // C is symmetric
+        C2[r * (m + 1) + c] = acc;
     }
     __syncthreads();
     for (int it = 0; it < PCA_ITERS; ++it) {
-        for (int i = t; i < m * PCA_D; i += blockDim.x) {   // W = C V, C = S / N - mu mu^T
-            const int r = i / PCA_D, d = i - r * PCA_D;
+        for (int i = t; i < m * PCA_D; i += blockDim.x) {
+            const int d = i / m, r = i - d * m;
             float acc = 0.f;
-            for (int c = 0; c < m; ++c) acc = fmaf(C[r * m + c], V[c][d], acc);
-            Wm[r][d] = acc;
+            for (int c = 0; c < m; ++c) acc = fmaf(C2[r * (m + 1) + c], V[d][c], acc);
+            Wm[d][r] = acc;
         }
         __syncthreads();
-        for (int d = 0; d < PCA_D; ++d) {   // Gram-Schmidt on column d against the earlier ones
-            for (int e = 0; e <= d; ++e) {
-                float part = 0.f;
-                for (int r = t; r < m; r += blockDim.x) part += (e < d ? V[r][e] : Wm[r][d]) * Wm[r][d];
+        if (w == 0) {
+            float v[PCA_D][4];   // rows lane, lane + 32, ...
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-                if (lane == 0) red[w] = part;
-                __syncthreads();
-                float dot = 0.f;
-                for (int q = 0; q < 8; ++q) dot += red[q];
-                __syncthreads();
-                if (e < d) {
-                    for (int r = t; r < m; r += blockDim.x) Wm[r][d] -= dot * V[r][e];
-                } else {
-                    const float inv = dot > 0.f ? rsqrtf(dot) : 0.f;
-                    for (int r = t; r < m; r += blockDim.x) V[r][d] = Wm[r][d] * inv;
+            for (int d = 0; d < PCA_D; ++d) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v[d][q] = lane + 32 * q < m ? Wm[d][lane + 32 * q] : 0.f;
+#pragma unroll
+                for (int e = 0; e <= d; ++e) {
+                    float dot = 0.f;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) dot = fmaf(v[e][q], v[d][q], dot);
+                    dot = warp_sum_f32(dot);
+                    const float f = dot > 0.f ? rsqrtf(dot) : 0.f;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v[d][q] = e < d ? v[d][q] - dot * v[e][q] : v[d][q] * f;
                 }
-                __syncthreads();
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (lane + 32 * q < m) V[d][lane + 32 * q] = v[d][q];
             }
         }
+        __syncthreads();
     }
     double* out = mom + 1 + m + (size_t)m * m;
-    for (int i = t; i < m * PCA_D; i += blockDim.x) out[i] = (double)V[i / PCA_D][i % PCA_D];
+    for (int i = t; i < m * PCA_D; i += blockDim.x) out[i] = (double)V[i % PCA_D][i / PCA_D];
 }
 
 // Projections of every point on the axes: proj[i][d] = sum_r x_ir V_rd.
@@ -387,18 +538,22 @@ __global__ void cloud_key_kernel(const uint32_t* __restrict__ val, int64_t n, Cl
     if (i < n) key[i] = (uint32_t)cloud_id(cl, (int64_t)val[i]);
 }
 
-__global__ void radix_hist_kernel(const uint32_t* __restrict__ key, int64_t n, int shift, uint32_t* hist, int nblk)
+// Digit counts of a block's `items` consecutive keys; layout [digit][block], or [block][digit] when the scatter sums
+// them itself.
+__global__ void radix_hist_kernel(const uint32_t* __restrict__ key, int64_t n, int shift, uint32_t* hist, int nblk,
+                                  int items, int fused)
 {
     __shared__ uint32_t cnt[256];
     cnt[threadIdx.x] = 0;
     __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * RADIX_ITEMS;
-    for (int r = 0; r < RADIX_ITEMS / RADIX_T; ++r) {
+    int64_t base = (int64_t)blockIdx.x * items;
+    for (int r = 0; r < items / RADIX_T; ++r) {
         int64_t e = base + r * RADIX_T + threadIdx.x;
         if (e < n) atomicAdd(&cnt[(key[e] >> shift) & 255u], 1u);
     }
     __syncthreads();
-    hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = cnt[threadIdx.x];
+    if (fused) hist[(int64_t)blockIdx.x * 256 + threadIdx.x] = cnt[threadIdx.x];
+    else hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = cnt[threadIdx.x];
 }
 
 // In-place exclusive scan of len uint32 values: per-block sums of 8192 values, one
@@ -499,14 +654,37 @@ static int scan_u32(cudaStream_t s, uint32_t* a, int64_t len, uint32_t* bsum)
 // round the order is (warp, lane), ranked with __match_any_sync.
 __global__ void radix_scatter_kernel(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
                                      uint32_t* kout, uint32_t* vout, int64_t n, int shift,
-                                     const uint32_t* __restrict__ hist, int nblk)
+                                     const uint32_t* __restrict__ hist, int nblk, int items, int fused)
 {
     __shared__ uint32_t base[256];
     __shared__ uint32_t wcnt[RADIX_T / 32][256];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    base[t] = hist[(int64_t)t * nblk + blockIdx.x];
-    int64_t b0 = (int64_t)blockIdx.x * RADIX_ITEMS;
-    for (int r = 0; r < RADIX_ITEMS / RADIX_T; ++r) {
+    if (fused) {
+        // few blocks: each adds up the counts before it (its digit in the blocks before, all smaller
+        // digits) instead of three scan launches
+        uint32_t mine = 0, all = 0;
+        for (int b = 0; b < nblk; ++b) {
+            const uint32_t c = hist[(int64_t)b * 256 + t];
+            if (b < (int)blockIdx.x) mine += c;
+            all += c;
+        }
+        __shared__ uint32_t wsum[RADIX_T / 32];
+        uint32_t inc = all;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) wsum[w] = inc;
+        __syncthreads();
+        uint32_t pre = inc - all;
+        for (int ww = 0; ww < w; ++ww) pre += wsum[ww];
+        base[t] = pre + mine;
+    } else {
+        base[t] = hist[(int64_t)t * nblk + blockIdx.x];
+    }
+    int64_t b0 = (int64_t)blockIdx.x * items;
+    for (int r = 0; r < items / RADIX_T; ++r) {
         for (int i = t; i < (RADIX_T / 32) * 256; i += RADIX_T) (&wcnt[0][0])[i] = 0;
         __syncthreads();
         int64_t e = b0 + r * RADIX_T + t;
@@ -2833,49 +3011,84 @@ static vb_status order_points(Ctx* ctx, const float* x, int64_t n, int32_t m, co
     cudaStream_t s = ctx->stream;
     const int mp = pad_dim(m), md = morton_dims(m), bits = morton_bits(md);
     const int64_t ntiles = (n + TILE - 1) / TILE, npad = (ntiles + (ntiles & 1)) * TILE;
-    const int nblk = (int)((n + RADIX_ITEMS - 1) / RADIX_ITEMS);
-    bbox_init_kernel<<<1, 32, 0, s>>>(w.bbox, w.fb_count);
+    const unsigned pt_grid = (unsigned)((n + 255) / 256);
     const unsigned bbox_grid = (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 4);
-    if (m <= 4) {
-        bbox_kernel<<<bbox_grid, 256, 0, s>>>(x, n, m, md, w.bbox, ctx->rep);
-        // the Hilbert curve at 2 <= m <= 4 unless the caller asks for the Morton curve
-        const int hilbert = curve == VB_CURVE_AUTO && md >= 2 ? 1 : 0;
-        morton_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, n, m, md, bits, w.bbox, w.key[0], w.val[0],
-                                                                  hilbert);
-    } else {
+    const bool small = n <= SMALL_N && mp <= 8 && cl.B <= 1;   // one block copies few coordinates
+    // the Hilbert curve at 2 <= m <= 4 unless the caller asks for the Morton curve
+    const int hilbert = m <= 4 && curve == VB_CURVE_AUTO && md >= 2 ? 1 : 0;
+    const float* kx = x;   // the rows that the keys are built on
+    int kld = m;
+    if (m > 4) {
         // finite check of the input, then the key on the leading principal axes
-        bbox_kernel<<<bbox_grid, 256, 0, s>>>(x, n, m, 0, w.bbox, ctx->rep);
+        finite_kernel<<<(unsigned)std::min<int64_t>((n * m + 255) / 256, 152 * 8), 256, 0, s>>>(x, n * m, ctx->rep);
         const int64_t stride = std::max<int64_t>(1, n / PCA_SAMPLE), rows = (n + stride - 1) / stride;
         const int64_t mlen = 1 + m + (int64_t)m * m;
+        const int csm = m * (m + 1) * (int)sizeof(float);
+        static bool attr_set[16] = {};
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (!attr_set[dev & 15]) {
+            if (cudaFuncSetAttribute(pca_axes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 129 * 4) !=
+                cudaSuccess)
+                return VB_ERR_CUDA;
+            attr_set[dev & 15] = true;
+        }
         pca_zero_kernel<<<(unsigned)((mlen + 255) / 256), 256, 0, s>>>(w.pcs, mlen);
         pca_moments_kernel<<<PCA_BLOCKS, 256, 0, s>>>(x, n, m, stride, rows, w.pcs);
-        pca_axes_kernel<<<1, 256, 0, s>>>(w.pcs, m, w.pcc);
-        pca_project_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, n, m, w.pcs + mlen, w.proj);
-        bbox_kernel<<<bbox_grid, 256, 0, s>>>(w.proj, n, PCA_D, PCA_D, w.bbox, ctx->rep);
-        morton_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(w.proj, n, PCA_D, PCA_D, bits, w.bbox, w.key[0],
-                                                                  w.val[0], 0);
-        ctx->launches += 5;   // moments zeroed, moments, axes, projection, box of the projections
+        pca_axes_kernel<<<1, 256, csm, s>>>(w.pcs, m, w.pcc);
+        pca_project_kernel<<<pt_grid, 256, 0, s>>>(x, n, m, w.pcs + mlen, w.proj);
+        ctx->launches += 5;   // finite check, moments zeroed, moments, axes, projection
+        kx = w.proj;
+        kld = PCA_D;
     }
+    if (small) {
+#define VB_SMALL(MD)                                                                                                  \
+    small_order_kernel<MD><<<1, SMALL_T, 0, s>>>(x, kx, kld, (int)n, (int)npad, m, mp, bits, hilbert, w.val[0], w.xs, \
+                                                 w.xs64, w.tlo, w.thi, w.slo, w.shi, w.fb_count, ctx->rep)
+        switch (md) {
+            case 1: VB_SMALL(1); break;
+            case 2: VB_SMALL(2); break;
+            case 3: VB_SMALL(3); break;
+            case 4: VB_SMALL(4); break;
+            default: VB_SMALL(5); break;
+        }
+#undef VB_SMALL
+        ctx->launches += 1;
+        *perm_out = w.val[0];
+        return last_launch();
+    }
+    bbox_init_kernel<<<1, 32, 0, s>>>(w.bbox, w.fb_count);
+#define VB_KEYS(MD)                                                                                        \
+    bbox_kernel<MD><<<bbox_grid, 256, 0, s>>>(kx, n, kld, w.bbox, ctx->rep);                               \
+    morton_kernel<MD><<<pt_grid, 256, 0, s>>>(kx, n, kld, bits, w.bbox, w.key[0], w.val[0], hilbert)
+    switch (md) {
+        case 1: VB_KEYS(1); break;
+        case 2: VB_KEYS(2); break;
+        case 3: VB_KEYS(3); break;
+        case 4: VB_KEYS(4); break;
+        default: VB_KEYS(5); break;
+    }
+#undef VB_KEYS
     int cur = 0;
-    for (int shift = 0; shift < 32; shift += 8) {
-        radix_hist_kernel<<<nblk, RADIX_T, 0, s>>>(w.key[cur], n, shift, w.hist, nblk);
-        ctx->launches += 2 + scan_u32(s, w.hist, (int64_t)256 * nblk, w.hsum);
-        radix_scatter_kernel<<<nblk, RADIX_T, 0, s>>>(w.key[cur], w.val[cur], w.key[cur ^ 1], w.val[cur ^ 1], n,
-                                                      shift, w.hist, nblk);
+    // smaller blocks while they stay few enough for the scatter to add up their counts itself
+    const int items = n <= 128 * 512 ? 512 : RADIX_ITEMS;
+    const int nblk = (int)((n + items - 1) / items), fused = nblk <= 128 ? 1 : 0;
+    auto radix_pass = [&](int shift) {
+        radix_hist_kernel<<<nblk, RADIX_T, 0, s>>>(w.key[cur], n, shift, w.hist, nblk, items, fused);
+        ctx->launches += 2 + (fused ? 0 : scan_u32(s, w.hist, (int64_t)256 * nblk, w.hsum));
+        radix_scatter_kernel<<<nblk, RADIX_T, 0, s>>>(w.key[cur], w.val[cur], w.key[cur ^ 1], w.val[cur ^ 1], n, shift,
+                                                      w.hist, nblk, items, fused);
         cur ^= 1;
-    }
+    };
+    // keys of md * bits bits; below 2^18 points the lowest eight would only order points inside cells far
+    // smaller than a tile
+    for (int shift = n < (1 << 18) && md * bits >= 30 ? 8 : 0; shift < md * bits; shift += 8) radix_pass(shift);
     if (cl.B > 1) {
         // stable passes on the cloud id: (cloud, Morton) order, so cloud b occupies the sorted
         // positions [ptr[b], ptr[b + 1]), the same range as its points in the input
-        cloud_key_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(w.val[cur], n, cl, w.key[cur]);
+        cloud_key_kernel<<<pt_grid, 256, 0, s>>>(w.val[cur], n, cl, w.key[cur]);
         ctx->launches += 1;
-        for (int shift = 0; (int64_t)(cl.B - 1) >> shift; shift += 8) {
-            radix_hist_kernel<<<nblk, RADIX_T, 0, s>>>(w.key[cur], n, shift, w.hist, nblk);
-            ctx->launches += 2 + scan_u32(s, w.hist, (int64_t)256 * nblk, w.hsum);
-            radix_scatter_kernel<<<nblk, RADIX_T, 0, s>>>(w.key[cur], w.val[cur], w.key[cur ^ 1], w.val[cur ^ 1], n,
-                                                          shift, w.hist, nblk);
-            cur ^= 1;
-        }
+        for (int shift = 0; (int64_t)(cl.B - 1) >> shift; shift += 8) radix_pass(shift);
     }
     const uint32_t* perm = w.val[cur];
     gather_kernel<<<(unsigned)((npad * mp + 255) / 256), 256, 0, s>>>(x, perm, n, npad, m, mp, w.xs, w.xs64);
