@@ -54,14 +54,14 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t* sh, int64
     return r;
 }
 
-__global__ void __launch_bounds__(SCAN_T) scan_reduce_kernel(const int32_t* __restrict__ c, int64_t n, int64_t* bsum)
+__global__ void __launch_bounds__(SCAN_T) scan_reduce_kernel(const int32_t* __restrict__ c, int64_t n, int add, int64_t* bsum)
 {
     __shared__ int64_t sh[32];
     int64_t base = (int64_t)blockIdx.x * SCAN_T * SCAN_ITEMS;
     int64_t s = 0;
     for (int i = 0; i < SCAN_ITEMS; ++i) {
         int64_t e = base + (int64_t)i * SCAN_T + threadIdx.x;
-        if (e < n) s += c[e];
+        if (e < n) s += c[e] + add;
     }
     int64_t tot;
     block_excl_scan(s, sh, &tot);
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(SCAN_T) scan_top_kernel(int64_t* bsum, int64_t
     if (threadIdx.x == 0) bsum[nb] = carry;
 }
 
-__global__ void __launch_bounds__(SCAN_T) scan_apply_kernel(const int32_t* __restrict__ c, int64_t n,
+__global__ void __launch_bounds__(SCAN_T) scan_apply_kernel(const int32_t* __restrict__ c, int64_t n, int add,
                                                            const int64_t* __restrict__ bsum, int64_t nb, int64_t* out)
 {
     __shared__ int64_t sh[32];
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(SCAN_T) scan_apply_kernel(const int32_t* __res
     int64_t s = 0;
 #pragma unroll
     for (int i = 0; i < SCAN_ITEMS; ++i) {
-        v[i] = base + i < n ? c[base + i] : 0;
+        v[i] = base + i < n ? c[base + i] + add : 0;
         s += v[i];
     }
     int64_t run = bsum[blockIdx.x] + block_excl_scan(s, sh, nullptr);
@@ -109,13 +109,13 @@ __global__ void __launch_bounds__(SCAN_T) scan_apply_kernel(const int32_t* __res
     if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = bsum[nb];
 }
 
-vb_status scan_counts(cudaStream_t s, const int32_t* counts, int64_t n, int64_t* out, void* ws)
+vb_status scan_counts(cudaStream_t s, const int32_t* counts, int64_t n, int64_t* out, void* ws, int add)
 {
     int64_t nb = (n + SCAN_T * SCAN_ITEMS - 1) / (SCAN_T * SCAN_ITEMS);
     int64_t* bsum = (int64_t*)ws;
-    scan_reduce_kernel<<<(unsigned)nb, SCAN_T, 0, s>>>(counts, n, bsum);
+    scan_reduce_kernel<<<(unsigned)nb, SCAN_T, 0, s>>>(counts, n, add, bsum);
     scan_top_kernel<<<1, SCAN_T, 0, s>>>(bsum, nb);
-    scan_apply_kernel<<<(unsigned)nb, SCAN_T, 0, s>>>(counts, n, bsum, nb, out);
+    scan_apply_kernel<<<(unsigned)nb, SCAN_T, 0, s>>>(counts, n, add, bsum, nb, out);
     return last_launch();
 }
 
@@ -126,12 +126,15 @@ vb_status scan_counts(cudaStream_t s, const int32_t* counts, int64_t n, int64_t*
 // in N(j), which for exact lists ordered by (d2, index) holds exactly when
 // (d2(i, j), i) <= (d2 and index of j's k-th neighbour), one 16-byte load instead of a
 // search, so mutual pairs enter once; the counts
-// 1 + k + |R(j)| give row_ptr directly (one scan); the kept reverse entries are
-// scattered into a side buffer; finally one warp per row sorts R(j) and places
-// every entry by its rank (own index + reverse entries below it + the diagonal),
+// 1 + k + |R(j)| give row_ptr directly (one scan).  A kept reverse entry goes straight into one of
+// row j's RBUCKET slots as it is counted; what overflows them is listed (and marked in the sorted list, for
+// when the list overflows too) and scattered behind row_ptr in a second pass.  Finally one warp per row sorts
+// R(j) and places every entry by its rank (own index + reverse entries below it + the diagonal),
 // which merges the three sorted sets with no duplicates left to remove.
 constexpr int RCAP = 256;           // warp path: reverse entries per row held in shared memory
 constexpr int OWN_CAP = 256;        // longest kNN list (k + margin <= 256)
+constexpr int RBUCKET = 32;         // reverse entries a row takes without the second pass
+constexpr int OVER_CAP = 1 << 16;   // entries beyond the buckets that are listed (more: every list is scanned)
 
 struct Kth {
     double d2;         // j's k-th neighbour distance and index
@@ -143,12 +146,13 @@ struct GraphWs {
     int32_t* own_col;  // n k: kNN lists sorted by column
     float* own_d2;     // n k
     int32_t* rcnt;     // n reverse entries per row
-    int32_t* fill;     // n scatter cursors
-    int32_t* cnt;      // n row lengths
-    int32_t* rev_col;  // n k reverse entries, row j at row_ptr[j] - j (1 + k)
+    int32_t* fill;     // n scatter cursors of the entries beyond RBUCKET
+    int2* bucket;      // n RBUCKET reverse entries (row, distance bits)
+    int32_t* rev_col;  // n k: those beyond RBUCKET, entry e of row j at row_ptr[j] - j (1 + k) + e
     float* rev_d2;     // n k
     int32_t* big;      // n rows for the block path
-    int32_t* nbig;     // 1
+    int32_t* nbig;     // [0] rows for the block path, [1] entries beyond RBUCKET
+    int4* over;        // OVER_CAP of those: (i, j, distance bits, -)
     void* scan;        // scan_ws_bytes(n)
 };
 
@@ -160,11 +164,12 @@ static size_t graph_plan(Carve& c, int64_t n, int32_t k, GraphWs* w)
     t.own_d2 = c.take<float>(n * (int64_t)k);
     t.rcnt = c.take<int32_t>(n);
     t.fill = c.take<int32_t>(n);
-    t.cnt = c.take<int32_t>(n);
+    t.bucket = c.take<int2>(n * RBUCKET);
     t.rev_col = c.take<int32_t>(n * (int64_t)k);
     t.rev_d2 = c.take<float>(n * (int64_t)k);
     t.big = c.take<int32_t>(n);
-    t.nbig = c.take<int32_t>(1);
+    t.nbig = c.take<int32_t>(2);
+    t.over = c.take<int4>(OVER_CAP);
     t.scan = c.take<char>(scan_ws_bytes(n));
     if (w) *w = t;
     return c.off;
@@ -173,12 +178,6 @@ size_t graph_plan_bytes(int64_t n, int32_t k)
 {
     Carve c(nullptr);
     return graph_plan(c, n, k, nullptr);
-}
-
-__global__ void zero_i32_kernel(int32_t* a, int64_t n)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        a[i] = 0;
 }
 
 // bitonic sort of P (power of two) 64-bit keys in shared memory by `nthr` threads
@@ -222,14 +221,17 @@ __device__ __forceinline__ int lower_bound_key(const uint64_t* a, int len, int32
 
 constexpr int SORT_WARPS = 4;
 
-// The k-th pair (distance, index) of every list, 16 bytes per point: the table the mutual
+// Clears the counters, and the k-th pair (distance, index) of every list, 16 bytes per point: the table the mutual
 // test below reads at random stays in L2, where the lists themselves (12 k bytes per point)
 // do not.
 __global__ void kth_kernel(const int32_t* __restrict__ nbr, const double* __restrict__ nbr_d2, int64_t n, int k,
-                           Kth* kth)
+                           Kth* kth, int32_t* rcnt, int32_t* fill, int32_t* nbig)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < 2) nbig[i] = 0;
     if (i >= n) return;
+    rcnt[i] = 0;
+    fill[i] = 0;
     Kth q;
     q.d2 = nbr_d2[i * k + k - 1];
     q.idx = nbr[i * k + k - 1];
@@ -238,138 +240,121 @@ __global__ void kth_kernel(const int32_t* __restrict__ nbr, const double* __rest
 }
 
 // Own kNN lists sorted by column, one warp per row; the FP32 value of each entry is the
-// rounding of its canonical FP64 distance (identical for (i, j) and (j, i)).  The columns of a
-// list are distinct, so an entry's place in the sorted list is the number of columns below its
-// own: every column is broadcast to the warp once (a shuffle) and each lane counts for the KL
-// entries it holds, then writes each entry straight to its place.  No shared memory: a
-// bitonic network over 64-bit keys in shared memory was bound by its shared-memory traffic.
-// The same pass counts, for every point j, the lists that name j without j naming their owner
-// (the reverse entries of row j): (i -> j) is mutual exactly when (d2(i, j), i) does not exceed
-// the k-th pair of j's own list (kth[j]).  A non-mutual entry carries the sign bit in own_d2
-// (distances are >= 0), so the scatter pass reads the sorted lists alone.
-// For k <= 64 and n <= 2^26 the list is instead sorted as 32-bit keys column << 6 | position
-// (columns distinct, so the order is the columns' order) by a bitonic network across the warp,
-// two keys per lane: 21 compare-exchange steps of one shuffle each instead of k broadcasts with
-// k compares, and each sorted key names the entry it came from.
-template <int KL>
-__device__ __forceinline__ void warp_bitonic(uint32_t (&key)[KL], int lane)
+// rounding of its canonical FP64 distance (identical for (i, j) and (j, i)).  The same pass finds, for
+// every point j, the lists that name j without j naming their owner (the reverse entries of row j):
+// (i -> j) is mutual exactly when (d2(i, j), i) does not exceed the k-th pair of j's own list
+// (kth[j]).  A non-mutual entry is counted and put into row j's bucket in one atomic; beyond
+// RBUCKET it is listed and carries the sign bit in own_d2 (distances are >= 0) for the second pass.  (Marking
+// all of them and scattering in a pass over every entry took 0.48 ms more at 1M torus points, k = 64.)
+// SORT: the list is sorted as 32-bit keys column << (5 + log2 KL) | position (columns distinct, so the order is
+// the columns' order) by a bitonic network across the warp, for k <= 32 KL <= 128 and columns that fit;
+// else an entry's place is the number of columns below its own: every column is broadcast to the warp
+// once and each lane counts for the KL entries it holds.
+__device__ __forceinline__ float own_entry(int64_t i, int32_t j, double d, int k, const Kth* __restrict__ kth,
+                                           int32_t* rcnt, int2* bucket, int32_t* nover, int4* over)
 {
-    constexpr int N = 32 * KL;
-#pragma unroll
-    for (int size = 2; size <= N; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride == 32) {   // N = 64: the partner is this lane's other key
-                const uint32_t a = key[0], b = key[KL - 1];
-                key[0] = min(a, b);
-                key[KL - 1] = max(a, b);
-            } else {
-#pragma unroll
-                for (int s = 0; s < KL; ++s) {
-                    const uint32_t o = __shfl_xor_sync(0xffffffffu, key[s], stride);
-                    const bool lower = (lane & stride) == 0, up = ((lane + 32 * s) & size) == 0;
-                    key[s] = lower == up ? min(key[s], o) : max(key[s], o);
-                }
-            }
-        }
+    const Kth q = kth[j];
+    const float f = (float)d;
+    if (d < q.d2 || (d == q.d2 && (int32_t)i <= q.idx)) return f;
+    const int slot = atomicAdd(&rcnt[j], 1);
+    if (slot < RBUCKET) {
+        bucket[(int64_t)j * RBUCKET + slot] = make_int2((int32_t)i, __float_as_int(f));
+        return f;
     }
+    const int at = atomicAdd(nover, 1);
+    if (at < OVER_CAP) over[at] = make_int4((int32_t)i, j, __float_as_int(f), 0);
+    return -f;
 }
 
-template <int KL>
+template <int KL, bool SORT>
 __global__ void __launch_bounds__(SORT_WARPS * 32) own_sort_kernel(const int32_t* __restrict__ nbr,
                                                                     const double* __restrict__ nbr_d2, int64_t n,
                                                                     int k, int32_t* own_col, float* own_d2,
-                                                                    const Kth* __restrict__ kth, int32_t* rcnt)
+                                                                    const Kth* __restrict__ kth, int32_t* rcnt,
+                                                                    int2* bucket, int32_t* nover, int4* over)
 {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if constexpr (KL <= 2) {
-        if (n <= ((int64_t)1 << 26)) {
-            for (int64_t i = (int64_t)blockIdx.x * SORT_WARPS + w; i < n; i += (int64_t)gridDim.x * SORT_WARPS) {
-                const int32_t* row = nbr + i * k;
-                uint32_t key[KL];
-#pragma unroll
-                for (int s = 0; s < KL; ++s) {
-                    const int e = lane + 32 * s;
-                    key[s] = e < k ? ((uint32_t)row[e] << 6) | (uint32_t)e : 0xffffffffu;
-                }
-                warp_bitonic<KL>(key, lane);
-#pragma unroll
-                for (int s = 0; s < KL; ++s) {
-                    const int pos = lane + 32 * s;   // the key's place in the sorted list
-                    if (pos < k) {
-                        const int32_t j = (int32_t)(key[s] >> 6);
-                        const int e = (int)(key[s] & 63u);
-                        const double d = nbr_d2[i * k + e];
-                        const Kth q = kth[j];
-                        const bool rev = !(d < q.d2 || (d == q.d2 && (int32_t)i <= q.idx));
-                        own_col[i * k + pos] = j;
-                        own_d2[i * k + pos] = rev ? -(float)d : (float)d;
-                        if (rev) atomicAdd(&rcnt[j], 1);
-                    }
-                }
-            }
-            return;
-        }
-    }
     for (int64_t i = (int64_t)blockIdx.x * SORT_WARPS + w; i < n; i += (int64_t)gridDim.x * SORT_WARPS) {
         const int32_t* row = nbr + i * k;
-        int32_t c[KL];
-        int rank[KL];
+        if constexpr (SORT) {
+            constexpr int PB = KL == 1 ? 5 : KL == 2 ? 6 : 7;
+            uint32_t key[KL];
 #pragma unroll
-        for (int s = 0; s < KL; ++s) {
-            const int e = lane + 32 * s;
-            c[s] = e < k ? row[e] : INT32_MAX;
-            rank[s] = 0;
-        }
-#pragma unroll
-        for (int s2 = 0; s2 < KL; ++s2) {
-            const int32_t v = c[s2];
-            const int lim = min(32, k - 32 * s2);
-            for (int l = 0; l < lim; ++l) {
-                const int32_t cb = __shfl_sync(0xffffffffu, v, l);
-#pragma unroll
-                for (int s = 0; s < KL; ++s) rank[s] += cb < c[s] ? 1 : 0;
+            for (int s = 0; s < KL; ++s) {
+                const int e = lane + 32 * s;
+                key[s] = e < k ? ((uint32_t)row[e] << PB) | (uint32_t)e : 0xffffffffu;
             }
-        }
+            warp_sort<KL>(key, lane);
 #pragma unroll
-        for (int s = 0; s < KL; ++s) {
-            const int e = lane + 32 * s;
-            if (e < k) {
-                const double d = nbr_d2[i * k + e];
-                const int32_t j = c[s];
-                const Kth q = kth[j];
-                const bool rev = !(d < q.d2 || (d == q.d2 && (int32_t)i <= q.idx));
-                own_col[i * k + rank[s]] = j;
-                own_d2[i * k + rank[s]] = rev ? -(float)d : (float)d;
-                if (rev) atomicAdd(&rcnt[j], 1);
+            for (int s = 0; s < KL; ++s) {
+                const int pos = lane * KL + s;   // the key's place in the sorted list
+                if (pos < k) {
+                    const int32_t j = (int32_t)(key[s] >> PB);
+                    const double d = nbr_d2[i * k + (key[s] & ((1u << PB) - 1u))];
+                    own_col[i * k + pos] = j;
+                    own_d2[i * k + pos] = own_entry(i, j, d, k, kth, rcnt, bucket, nover, over);
+                }
+            }
+        } else {
+            int32_t c[KL];
+            int rank[KL];
+#pragma unroll
+            for (int s = 0; s < KL; ++s) {
+                const int e = lane + 32 * s;
+                c[s] = e < k ? row[e] : INT32_MAX;
+                rank[s] = 0;
+            }
+#pragma unroll
+            for (int s2 = 0; s2 < KL; ++s2) {
+                const int32_t v = c[s2];
+                const int lim = min(32, k - 32 * s2);
+                for (int l = 0; l < lim; ++l) {
+                    const int32_t cb = __shfl_sync(0xffffffffu, v, l);
+#pragma unroll
+                    for (int s = 0; s < KL; ++s) rank[s] += cb < c[s] ? 1 : 0;
+                }
+            }
+#pragma unroll
+            for (int s = 0; s < KL; ++s) {
+                const int e = lane + 32 * s;
+                if (e < k) {
+                    own_col[i * k + rank[s]] = c[s];
+                    own_d2[i * k + rank[s]] = own_entry(i, c[s], nbr_d2[i * k + e], k, kth, rcnt, bucket, nover, over);
+                }
             }
         }
     }
 }
 
-// The non-mutual entries (i -> j) of the sorted lists (sign bit set in own_d2), scattered
-// into row j's reverse slots.
+// The entries (i -> j) beyond row j's bucket, from the list, or all with the sign bit set in own_d2,
+// scattered behind row_ptr.
 __global__ void reverse_kernel(const int32_t* __restrict__ own_col, const float* __restrict__ own_d2, int64_t n, int k,
-                               const int64_t* __restrict__ row_ptr, int32_t* fill, int32_t* rev_col, float* rev_d2)
+                               const int64_t* __restrict__ row_ptr, int32_t* fill, int32_t* rev_col, float* rev_d2,
+                               const int32_t* __restrict__ nover, const int4* __restrict__ over)
 {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= n * k) return;
-    const float d = own_d2[e];
-    if (!signbit(d)) return;   // mutual: already in row j's own list
-    const int64_t i = e / k;
-    const int32_t j = own_col[e];
-    const int slot = atomicAdd(&fill[j], 1);
-    const int64_t off = row_ptr[j] - (int64_t)j * (1 + k) + slot;
-    rev_col[off] = (int32_t)i;
-    rev_d2[off] = -d;
-}
-
-__global__ void row_len_kernel(const int32_t* __restrict__ rcnt, int64_t n, int k, int32_t* cnt, int32_t* fill)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) {
-        cnt[i] = 1 + k + rcnt[i];
-        fill[i] = 0;
+    const int no = *nover;
+    if (no == 0) return;
+    if (no <= OVER_CAP) {
+        for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < no; e += gridDim.x * blockDim.x) {
+            const int4 v = over[e];
+            const int64_t off = row_ptr[v.y] - (int64_t)v.y * (1 + k) + RBUCKET + atomicAdd(&fill[v.y], 1);
+            rev_col[off] = v.x;
+            rev_d2[off] = __int_as_float(v.z);
+        }
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    const int64_t step = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < n; i += step) {   // a warp per list
+        for (int e = lane; e < k; e += 32) {
+            const float d = own_d2[i * k + e];
+            if (!signbit(d)) continue;
+            const int32_t j = own_col[i * k + e];
+            const int slot = RBUCKET + atomicAdd(&fill[j], 1);
+            const int64_t off = row_ptr[j] - (int64_t)j * (1 + k) + slot;
+            rev_col[off] = (int32_t)i;
+            rev_d2[off] = -d;
+        }
     }
 }
 
@@ -378,14 +363,21 @@ __global__ void row_len_kernel(const int32_t* __restrict__ rcnt, int64_t n, int 
 // global memory (the block path).
 __device__ void merge_row(int64_t j, int k, int r, uint64_t* rb, const int64_t* __restrict__ row_ptr,
                           const int32_t* __restrict__ own_col, const float* __restrict__ own_d2,
-                          const int32_t* __restrict__ rev_col, const float* __restrict__ rev_d2, int32_t* col,
-                          float* ed2, int tid, int nthr, bool warp_only, int32_t* oc_s = nullptr)
+                          const int2* __restrict__ bucket, const int32_t* __restrict__ rev_col,
+                          const float* __restrict__ rev_d2, int32_t* col, float* ed2, int tid, int nthr,
+                          bool warp_only, int32_t* oc_s = nullptr)
 {
     int P = 32;
     while (P < r) P <<= 1;
     const int64_t roff = row_ptr[j] - j * (1 + k);
-    for (int e = tid; e < P; e += nthr)
-        rb[e] = e < r ? ((uint64_t)(uint32_t)rev_col[roff + e] << 32) | __float_as_uint(rev_d2[roff + e]) : ~0ull;
+    for (int e = tid; e < P; e += nthr) {
+        if (e < min(r, RBUCKET)) {
+            const int2 v = bucket[j * RBUCKET + e];
+            rb[e] = ((uint64_t)(uint32_t)v.x << 32) | (uint32_t)v.y;
+        } else {
+            rb[e] = e < r ? ((uint64_t)(uint32_t)rev_col[roff + e] << 32) | __float_as_uint(rev_d2[roff + e]) : ~0ull;
+        }
+    }
     const int32_t* oc = own_col + j * k;
     if (oc_s) {   // the own columns, searched once per reverse entry, from shared memory
         for (int e = tid; e < k; e += nthr) oc_s[e] = oc[e];
@@ -422,15 +414,14 @@ __device__ void merge_row(int64_t j, int k, int r, uint64_t* rb, const int64_t* 
 template <int OWN_PER_LANE>   // own-list entries per lane: k <= 32 OWN_PER_LANE
 __device__ void merge_row_small(int64_t j, int k, int r, const int64_t* __restrict__ row_ptr,
                                 const int32_t* __restrict__ own_col, const float* __restrict__ own_d2,
-                                const int32_t* __restrict__ rev_col, const float* __restrict__ rev_d2, int32_t* col,
-                                float* ed2, int lane, int32_t* oc_s)
+                                const int2* __restrict__ bucket, int32_t* col, float* ed2, int lane, int32_t* oc_s)
 {
-    const int64_t roff = row_ptr[j] - j * (1 + k);
     int32_t rc = INT32_MAX;
     float rd = 0.f;
     if (lane < r) {
-        rc = rev_col[roff + lane];
-        rd = rev_d2[roff + lane];
+        const int2 v = bucket[j * RBUCKET + lane];
+        rc = v.x;
+        rd = __int_as_float(v.y);
     }
     const int32_t* oc = own_col + j * k;
     int32_t c[OWN_PER_LANE];
@@ -478,6 +469,7 @@ template <int KL>   // own-list entries per lane, k <= 32 KL
 __global__ void __launch_bounds__(SORT_WARPS * 32) merge_kernel(const int64_t* __restrict__ row_ptr, int64_t n, int k,
                                                                  const int32_t* __restrict__ own_col,
                                                                  const float* __restrict__ own_d2,
+                                                                 const int2* __restrict__ bucket,
                                                                  const int32_t* __restrict__ rev_col,
                                                                  const float* __restrict__ rev_d2, int32_t* col,
                                                                  float* ed2, int64_t cap, int32_t* big, int32_t* nbig,
@@ -500,10 +492,10 @@ __global__ void __launch_bounds__(SORT_WARPS * 32) merge_kernel(const int64_t* _
             }
             continue;
         }
-        if (r <= 32)
-            merge_row_small<KL>(j, k, r, row_ptr, own_col, own_d2, rev_col, rev_d2, col, ed2, lane, ocs[w]);
+        if (r <= RBUCKET)
+            merge_row_small<KL>(j, k, r, row_ptr, own_col, own_d2, bucket, col, ed2, lane, ocs[w]);
         else
-            merge_row(j, k, r, buf[w], row_ptr, own_col, own_d2, rev_col, rev_d2, col, ed2, lane, 32, true, ocs[w]);
+            merge_row(j, k, r, buf[w], row_ptr, own_col, own_d2, bucket, rev_col, rev_d2, col, ed2, lane, 32, true, ocs[w]);
         __syncwarp();
     }
 }
@@ -511,6 +503,7 @@ __global__ void __launch_bounds__(SORT_WARPS * 32) merge_kernel(const int64_t* _
 __global__ void __launch_bounds__(1024) big_merge_kernel(const int64_t* __restrict__ row_ptr, int64_t n, int k,
                                                         const int32_t* __restrict__ own_col,
                                                         const float* __restrict__ own_d2,
+                                                        const int2* __restrict__ bucket,
                                                         const int32_t* __restrict__ rev_col,
                                                         const float* __restrict__ rev_d2, int32_t* col, float* ed2,
                                                         int64_t cap, const int32_t* __restrict__ big,
@@ -526,7 +519,7 @@ __global__ void __launch_bounds__(1024) big_merge_kernel(const int64_t* __restri
             if (threadIdx.x == 0) report_error(rep, VB_ERR_UNSUPPORTED);
             continue;
         }
-        merge_row(j, k, r, bbuf, row_ptr, own_col, own_d2, rev_col, rev_d2, col, ed2, threadIdx.x, blockDim.x, false);
+        merge_row(j, k, r, bbuf, row_ptr, own_col, own_d2, bucket, rev_col, rev_d2, col, ed2, threadIdx.x, blockDim.x, false);
         __syncthreads();
     }
 }
@@ -542,41 +535,36 @@ vb_status graph_run(Ctx* ctx, int64_t n, int32_t k, const int32_t* nbr, const do
     size_t need = graph_plan(c, n, k, &w);
     if (!ws || ws_bytes < need) return VB_ERR_WORKSPACE;
     cudaStream_t s = ctx->stream;
-    const int64_t nk = n * k;
-    const unsigned gz = (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8);
-    const unsigned ge = (unsigned)((nk + 255) / 256);
     mark(ctx, VB_STAGE_GRAPH, 0);
-    zero_i32_kernel<<<gz, 256, 0, s>>>(w.rcnt, n);
-    zero_i32_kernel<<<1, 32, 0, s>>>(w.nbig, 1);
-    kth_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(nbr, nbr_d2, n, k, w.kth);
-    if (k <= 32)
-        own_sort_kernel<1><<<152 * 16, SORT_WARPS * 32, 0, s>>>(nbr, nbr_d2, n, k, w.own_col, w.own_d2, w.kth,
-                                                                   w.rcnt);
-    else if (k <= 64)
-        own_sort_kernel<2><<<152 * 16, SORT_WARPS * 32, 0, s>>>(nbr, nbr_d2, n, k, w.own_col, w.own_d2, w.kth,
-                                                                   w.rcnt);
-    else if (k <= 128)
-        own_sort_kernel<4><<<152 * 16, SORT_WARPS * 32, 0, s>>>(nbr, nbr_d2, n, k, w.own_col, w.own_d2, w.kth,
-                                                                   w.rcnt);
-    else
-        own_sort_kernel<8><<<152 * 16, SORT_WARPS * 32, 0, s>>>(nbr, nbr_d2, n, k, w.own_col, w.own_d2, w.kth,
-                                                                   w.rcnt);
-    row_len_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(w.rcnt, n, k, w.cnt, w.fill);
-    vb_status st = scan_counts(s, w.cnt, n, row_ptr, w.scan);
+    int32_t* nover = w.nbig + 1;
+    kth_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(nbr, nbr_d2, n, k, w.kth, w.rcnt, w.fill, w.nbig);
+    // sorted by keys of a column and a position while those fit 32 bits, else ranked by counting
+    const int pb = k <= 32 ? 5 : k <= 64 ? 6 : 7;
+    const bool keys = k <= 128 && n <= (int64_t)1 << (32 - pb);
+#define VB_OWN(KL, SORT)                                                                                            \
+    own_sort_kernel<KL, SORT><<<152 * 16, SORT_WARPS * 32, 0, s>>>(nbr, nbr_d2, n, k, w.own_col, w.own_d2, w.kth,     \
+                                                                w.rcnt, w.bucket, nover, w.over)
+    if (k <= 32) {
+        if (keys) VB_OWN(1, true); else VB_OWN(1, false);
+    } else if (k <= 64) {
+        if (keys) VB_OWN(2, true); else VB_OWN(2, false);
+    } else if (k <= 128) {
+        if (keys) VB_OWN(4, true); else VB_OWN(4, false);
+    } else {
+        VB_OWN(8, false);
+    }
+#undef VB_OWN
+    vb_status st = scan_counts(s, w.rcnt, n, row_ptr, w.scan, 1 + k);
     if (st != VB_OK) return st;
-    reverse_kernel<<<ge, 256, 0, s>>>(w.own_col, w.own_d2, n, k, row_ptr, w.fill, w.rev_col, w.rev_d2);
-    if (k <= 32)
-        merge_kernel<1><<<152 * 16, SORT_WARPS * 32, 0, s>>>(row_ptr, n, k, w.own_col, w.own_d2, w.rev_col, w.rev_d2, col, ed2,
-                                                      cap, w.big, w.nbig, nnz_dev, ctx->rep);
-    else if (k <= 64)
-        merge_kernel<2><<<152 * 16, SORT_WARPS * 32, 0, s>>>(row_ptr, n, k, w.own_col, w.own_d2, w.rev_col, w.rev_d2, col, ed2,
-                                                      cap, w.big, w.nbig, nnz_dev, ctx->rep);
-    else if (k <= 128)
-        merge_kernel<4><<<152 * 16, SORT_WARPS * 32, 0, s>>>(row_ptr, n, k, w.own_col, w.own_d2, w.rev_col, w.rev_d2, col, ed2,
-                                                      cap, w.big, w.nbig, nnz_dev, ctx->rep);
-    else
-        merge_kernel<OWN_CAP / 32><<<152 * 16, SORT_WARPS * 32, 0, s>>>(row_ptr, n, k, w.own_col, w.own_d2, w.rev_col, w.rev_d2, col, ed2,
-                                                      cap, w.big, w.nbig, nnz_dev, ctx->rep);
+    reverse_kernel<<<152 * 8, 256, 0, s>>>(w.own_col, w.own_d2, n, k, row_ptr, w.fill, w.rev_col, w.rev_d2, nover, w.over);
+#define VB_MERGE(KL)                                                                                                 \
+    merge_kernel<KL><<<152 * 16, SORT_WARPS * 32, 0, s>>>(row_ptr, n, k, w.own_col, w.own_d2, w.bucket, w.rev_col,      \
+                                                         w.rev_d2, col, ed2, cap, w.big, w.nbig, nnz_dev, ctx->rep)
+    if (k <= 32) VB_MERGE(1);
+    else if (k <= 64) VB_MERGE(2);
+    else if (k <= 128) VB_MERGE(4);
+    else VB_MERGE(OWN_CAP / 32);
+#undef VB_MERGE
     static bool big_attr[16] = {};
     int dev = ctx->device & 15;
     if (!big_attr[dev]) {
@@ -585,10 +573,10 @@ vb_status graph_run(Ctx* ctx, int64_t n, int32_t k, const int32_t* nbr, const do
             return VB_ERR_CUDA;
         big_attr[dev] = true;
     }
-    big_merge_kernel<<<152, 1024, BIG_CAP * 8, s>>>(row_ptr, n, k, w.own_col, w.own_d2, w.rev_col, w.rev_d2, col, ed2,
+    big_merge_kernel<<<152, 1024, BIG_CAP * 8, s>>>(row_ptr, n, k, w.own_col, w.own_d2, w.bucket, w.rev_col, w.rev_d2, col, ed2,
                                                     cap, w.big, w.nbig, ctx->rep);
     mark(ctx, VB_STAGE_GRAPH, 1);
-    ctx->launches += 12;
+    ctx->launches += 8;
     return last_launch();
 }
 

@@ -63,54 +63,6 @@ template <int SB> __device__ __forceinline__ float ws_lo(uint32_t key)
     return __uint_as_float((key & ~((1u << SB) - 1u)) >> 1);
 }
 
-// Ascending bitonic sort of 32 R keys, element e in lane e / R, register e % R: strides below R
-// stay inside a lane, so a sort of 128 takes 15 shuffle steps instead of 25.  Each merge starts with
-// the reversed exchange (e with e ^ (size - 1)), so every exchange puts the smaller key first.
-template <int R>
-__device__ __forceinline__ void ws_sort(uint32_t (&key)[R], int lane)
-{
-    constexpr int N = 32 * R;
-#pragma unroll
-    for (int size = 2; size <= N; size <<= 1) {
-        if (size <= R) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int q = r ^ (size - 1);
-                if (q < r) continue;
-                const uint32_t x = key[r], y = key[q];
-                key[r] = min(x, y);
-                key[q] = max(x, y);
-            }
-        } else {
-            const bool first = (lane & (size / R / 2)) == 0;
-            uint32_t o[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) o[r] = __shfl_xor_sync(0xffffffffu, key[R - 1 - r], size / R - 1);
-#pragma unroll
-            for (int r = 0; r < R; ++r) key[r] = (o[r] < key[r]) == first ? o[r] : key[r];
-        }
-#pragma unroll
-        for (int stride = size >> 2; stride > 0; stride >>= 1) {
-            if (stride >= R) {
-                const bool first = (lane & (stride / R)) == 0;
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const uint32_t o = __shfl_xor_sync(0xffffffffu, key[r], stride / R);
-                    key[r] = (o < key[r]) == first ? o : key[r];
-                }
-            } else {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    if (r & stride) continue;
-                    const uint32_t x = key[r], y = key[r | stride];
-                    key[r] = min(x, y);
-                    key[r | stride] = max(x, y);
-                }
-            }
-        }
-    }
-}
-
 // Sorts keys[0 .. cnt) (cnt <= 32 R) in place; the first ns ranks are written back.
 template <int R>
 __device__ __forceinline__ void ws_sort_keys(uint32_t* keys, int cnt, int ns, int lane)
@@ -121,7 +73,7 @@ __device__ __forceinline__ void ws_sort_keys(uint32_t* keys, int cnt, int ns, in
         const int e = r * 32 + lane;
         key[r] = e < cnt ? keys[e] : ~0u;
     }
-    ws_sort<R>(key, lane);
+    warp_sort<R>(key, lane);
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < R; ++r)
@@ -441,9 +393,9 @@ __global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn
                 }
             };
             auto nrows = [&](int u) { return (int)((at[u] - base[u]) >> 8); };
-            // this lane's candidates of tile ct: rotated from tile to tile, as a far query finds its
-            // neighbours at the same end of many tiles
-            auto first_of = [&](int ct) { return ct * TILE + ((lane + 11 * ct) & 31); };
+            // this lane's candidates of tile ct: rotated by a hash of the tile, as a far query finds its
+            // neighbours at the same end of many tiles, of those at the corners of the curve's cells
+            auto first_of = [&](int ct) { return ct * TILE + (int)((lane + ((uint32_t)ct * 2654435769u >> 27)) & 31u); };
             auto load_tile = [&](int ct, float4 (&v)[2][MP / 4]) {
                 const float4* row = (const float4*)(a.xs + (int64_t)first_of(ct) * MP);
 #pragma unroll

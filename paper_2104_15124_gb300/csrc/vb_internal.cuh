@@ -97,6 +97,54 @@ __device__ __forceinline__ float lg2_approx(float x)
 // x^y = 2^(y log2 x) for x > 0 on the SFU; relative error about |y log2 x| 2^-22.
 __device__ __forceinline__ float pow_sfu(float x, float y) { return ex2_approx(y * lg2_approx(x)); }
 
+// Ascending bitonic sort of 32 R keys, element e in lane e / R, register e % R: strides below R
+// stay inside a lane, so a sort of 128 takes 15 shuffle steps instead of 25.  Each merge starts with
+// the reversed exchange (e with e ^ (size - 1)), so every exchange puts the smaller key first.
+template <int R>
+__device__ __forceinline__ void warp_sort(uint32_t (&key)[R], int lane)
+{
+    constexpr int N = 32 * R;
+#pragma unroll
+    for (int size = 2; size <= N; size <<= 1) {
+        if (size <= R) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int q = r ^ (size - 1);
+                if (q < r) continue;
+                const uint32_t x = key[r], y = key[q];
+                key[r] = min(x, y);
+                key[q] = max(x, y);
+            }
+        } else {
+            const bool first = (lane & (size / R / 2)) == 0;
+            uint32_t o[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) o[r] = __shfl_xor_sync(0xffffffffu, key[R - 1 - r], size / R - 1);
+#pragma unroll
+            for (int r = 0; r < R; ++r) key[r] = (o[r] < key[r]) == first ? o[r] : key[r];
+        }
+#pragma unroll
+        for (int stride = size >> 2; stride > 0; stride >>= 1) {
+            if (stride >= R) {
+                const bool first = (lane & (stride / R)) == 0;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const uint32_t o = __shfl_xor_sync(0xffffffffu, key[r], stride / R);
+                    key[r] = (o < key[r]) == first ? o : key[r];
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if (r & stride) continue;
+                    const uint32_t x = key[r], y = key[r | stride];
+                    key[r] = min(x, y);
+                    key[r | stride] = max(x, y);
+                }
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------------------ point clouds of a batched build
 // Cloud b holds the points [ptr[b], ptr[b + 1]) (device array of B + 1 entries);
 // B == 1 with ptr == nullptr is the single cloud [0, n).
@@ -230,7 +278,8 @@ vb_status evolve_update_launch(cudaStream_t s, const float* x, int64_t n, int m,
 
 // exclusive scan of n int32 counts into n + 1 int64 offsets (graph.cu)
 size_t scan_ws_bytes(int64_t n);
-vb_status scan_counts(cudaStream_t s, const int32_t* counts, int64_t n, int64_t* out, void* ws);
+// (plus `add` each)
+vb_status scan_counts(cudaStream_t s, const int32_t* counts, int64_t n, int64_t* out, void* ws, int add = 0);
 
 inline vb_status cuda_status(cudaError_t e) { return e == cudaSuccess ? VB_OK : VB_ERR_CUDA; }
 inline vb_status last_launch() { return cuda_status(cudaGetLastError()); }
