@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(1024) sweep_finish_kernel(const double* __rest
                                                            const double* __restrict__ xi_c_dev, int warn_bit,
                                                            double* eps2, double* chi, double* dim, DevReport* rep)
 {
-    __shared__ double sh[kMaxGrid], lg[kMaxGrid];
+    __shared__ double sh[kMaxGrid], lg[kMaxGrid], ex[kMaxGrid];
     __shared__ double part[SEG_PARTS * SEG_COLS];
     const int b = blockIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -426,7 +426,14 @@ __global__ void __launch_bounds__(1024) sweep_finish_kernel(const double* __rest
         chi[(int64_t)b * G + threadIdx.x] = sh[threadIdx.x];
     }
     __syncthreads();
-    if (threadIdx.x < G) lg[threadIdx.x] = log(sh[threadIdx.x]);
+    // logs, and beside them eps^2 of every grid point (a chain of FP64 operations less at the end)
+    if (threadIdx.x < G) {
+        lg[threadIdx.x] = log(sh[threadIdx.x]);
+    } else if (threadIdx.x >= 512 && threadIdx.x < 512 + G) {
+        const int h = threadIdx.x - 512;
+        const double xc = xi_c_dev ? xi_c_dev[b] : 0.0;
+        ex[h] = exp2(xc + xi_lo + h * dxi);
+    }
     __syncthreads();
     if (w == 0) {
         const double inv = 1.0 / (dxi * 0.69314718055994531);
@@ -443,8 +450,7 @@ __global__ void __launch_bounds__(1024) sweep_finish_kernel(const double* __rest
             if (ov > bv || (ov == bv && ob < best)) { bv = ov; best = ob; }
         }
         if (lane == 0) {
-            const double xc = xi_c_dev ? xi_c_dev[b] : 0.0;
-            eps2[b] = exp2(xc + xi_lo + best * dxi);
+            eps2[b] = ex[best];
             dim[b] = 2.0 * bv;
             if (best == 0 || best == G - 2) atomicOr(&rep->warnings, warn_bit);
         }
