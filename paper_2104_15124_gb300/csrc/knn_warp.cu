@@ -393,9 +393,10 @@ __global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn
                 }
             };
             auto nrows = [&](int u) { return (int)((at[u] - base[u]) >> 8); };
+            uint32_t hash = 2654435769u;
             // this lane's candidates of tile ct: rotated by a hash of the tile, as a far query finds its
             // neighbours at the same end of many tiles, of those at the corners of the curve's cells
-            auto first_of = [&](int ct) { return ct * TILE + (int)((lane + ((uint32_t)ct * 2654435769u >> 27)) & 31u); };
+            auto first_of = [&](int ct) { return ct * TILE + (int)((lane + ((uint32_t)ct * hash >> 27)) & 31u); };
             auto load_tile = [&](int ct, float4 (&v)[2][MP / 4]) {
                 const float4* row = (const float4*)(a.xs + (int64_t)first_of(ct) * MP);
 #pragma unroll
@@ -573,13 +574,22 @@ __global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn
                     tmax[u] = fminf(pmax[u], r2q[u]);
                     thr[u] = (todo >> u & 1) ? fminf(guess, tmax[u]) : -1.f;
                 }
-                int np = 0;
+                int np = 0, tries = 0;
                 while (todo) {
                     const float tried[2] = {thr[0], thr[1]};
                     at[0] = base[0];
                     at[1] = base[1];
                     scan(todo != 1);
-                    if (full) return false;
+                    if (full) {
+                        // one lane's list ran out (a few rows in a million): once more with the candidates dealt
+                        // to other lanes; ties fill every lane's
+                        if (tries++ == 2) return false;
+                        hash = hash * 747796405u + 2891336452u | 1u;
+                        full = false;
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) thr[u] = (todo >> u & 1) ? tried[u] : -1.f;
+                        continue;
+                    }
                     __syncwarp();
                     int got = 0;
 #pragma unroll 1
