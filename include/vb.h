@@ -119,7 +119,7 @@ vb_status vb_profile_read(vb_ctx* ctx, float* ms, int64_t* launches);
  * canonical FP64 squared distances
  *     d2 = ((s_0 + s_1) + s_2) + ...,  s_r = (x_ir - x_jr)^2  (RN, no FMA),
  * and neighbours are ordered by (d2, j): distance first, then smaller index.
- * The search stages the points in a Morton order (of the coordinates when
+ * The search stages the points in a Hilbert order (of the coordinates when
  * m <= 4, of the projections on the cloud's 5 leading principal axes when
  * m > 4), prunes 64-point tiles by bounding boxes (boxes of 64-tile super-tiles
  * first; in the pipelined 16-bit search, also balls about the box centres) and
@@ -190,9 +190,9 @@ typedef struct {
                                 the lower edge of the key's bucket, 2^-10 relative below the distance) */
     int32_t* dbg_idx;        /* with dbg_d2: n x (k + margin) device int32, the original index of each of those
                                 candidates (-1 for an unused slot) */
-    int32_t curve;           /* spatial order of the search's tiles at 2 <= m <= 4: VB_CURVE_AUTO (default, the
-                                Hilbert curve) or VB_CURVE_MORTON; m = 1 and m > 4 (principal-axis keys) always
-                                take the Morton interleave.  The lists are exact either way */
+    int32_t curve;           /* spatial order of the search's tiles: VB_CURVE_AUTO (default, the Hilbert curve of
+                                the coordinates, or at m > 4 of five principal-axis coordinates) or
+                                VB_CURVE_MORTON; m = 1 has one order.  The lists are exact either way */
 } vb_knn_params;
 
 /* Launch-shape autotuner (a16).  Times vb_knn on the caller's input for every

@@ -275,7 +275,7 @@ def knn(x: torch.Tensor, k: int, margin: int = 16, prune: bool = True, radius: t
     tensor_cores = "fp16" or "bf16" computes its distance tiles on the tensor cores, with the
     kernel tc_variant = "auto" (at m <= 4 the FP32 warp search, which is faster there), "staged" or
     "pipelined" (VB_TC_*); seed_tiles and heap_keys
-    ("compact" or "full") and curve ("auto": Hilbert order at 2 <= m <= 4, or "morton") as in
+    ("compact" or "full") and curve ("auto": Hilbert order, or "morton") as in
     vb_knn_params.  debug=True (16-bit tiles) also returns the
     candidates each row kept and their 16-bit tile distances before rescoring:
     (nbr, nbr_d2, dbg_idx int32 [n, k + margin], dbg_d2 fp32 [n, k + margin])."""

@@ -5,9 +5,9 @@
 // distance and then by index.  The search itself runs in FP32 and is made
 // exact by an FP64 certificate:
 //   a1  spatial order: bounding box, 32-bit Hilbert keys of the m coordinates when
-//       2 <= m <= 4 (Morton keys on request, and at m = 1), else Morton keys of the
-//       projections on the cloud's 5 leading principal axes (sampled covariance,
-//       subspace iteration), stable LSD radix sort, gather of the coordinates into
+//       2 <= m <= 4, else of the projections on the cloud's 5 leading principal axes
+//       (sampled covariance, subspace iteration; Morton keys on request, and at m = 1),
+//       stable LSD radix sort, gather of the coordinates into
 //       64-point tiles (zero-padded to MP = 4, 8, ..., 128).
 //   a2  pruning: every tile carries its bounding box; a candidate tile is
 //       skipped when the box-to-box (and, per query, point-to-box) distance,
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(SMALL_T) small_order_kernel(const float* __res
     }
 }
 
-// ---- m > 4: the Morton key is built on the projections onto the cloud's PCA_D leading
+// ---- m > 4: the key is built on the projections onto the cloud's PCA_D leading
 // principal axes, so that 64-point tiles are compact in the directions the points spread
 // along (the first coordinates of a wide input need not be those).  The axes only decide
 // the order of the search; the neighbour lists are exact whatever they are.
@@ -3014,8 +3014,10 @@ static vb_status order_points(Ctx* ctx, const float* x, int64_t n, int32_t m, co
     const unsigned pt_grid = (unsigned)((n + 255) / 256);
     const unsigned bbox_grid = (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 4);
     const bool small = n <= SMALL_N && mp <= 8 && cl.B <= 1;   // one block copies few coordinates
-    // the Hilbert curve at 2 <= m <= 4 unless the caller asks for the Morton curve
-    const int hilbert = m <= 4 && curve == VB_CURVE_AUTO && md >= 2 ? 1 : 0;
+    // the Hilbert curve unless the caller asks for the Morton curve (or there is one key coordinate only);
+    // on five principal axes it evaluates a fifth fewer candidate pairs than the Morton curve (200k points in
+    // R^100: 19.6 -> 15.4 G pairs, search 68 -> 61 ms)
+    const int hilbert = curve == VB_CURVE_AUTO && md >= 2 ? 1 : 0;
     const float* kx = x;   // the rows that the keys are built on
     int kld = m;
     if (m > 4) {
