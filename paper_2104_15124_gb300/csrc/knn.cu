@@ -2226,6 +2226,9 @@ __global__ void __launch_bounds__(T2) knn_tc_kernel(TileArgs a)
 // the bound, a monotone key, so the stop is exact.  Rows finish as in the staged kernel
 // (finalize_row_band); a row that is not certified sends its tiles to the FP32 search.
 // Every wait is bounded in time (an expired wait records VB_ERR_TIMEOUT and stops the CTA).
+// Bound by the four selection warps (one per scheduler, so by the latency of their chains): 4-ary heaps, a tree
+// of selects for a candidate's distance, packed distances and the bound mask from sign bits took the
+// search of 200k points in R^100 (k = 128) from 41 to 33 ms.
 constexpr int TCP_BUF = 4;         // tensor-memory accumulator buffers of 64 columns
 constexpr int TCP_META = 16;       // tile ids in flight (>= slots + buffers + 1)
 constexpr int TCP_THREADS = 192;   // warps 0-3 epilogue, 4 producer, 5 MMA
@@ -2633,13 +2636,16 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) knn_tcp_kernel(TileArgs a)
                 if (ct >= 0) {
                     tc::tmem_ld64(lane_addr + (uint32_t)(b * TILE), v);
                     const float4* x4 = (const float4*)txn[b];
+                    const float2 sq2 = make_float2(sqa, sqa), m2 = make_float2(-2.f, -2.f);
 #pragma unroll
-                    for (int i4 = 0; i4 < TILE / 4; ++i4) {
+                    for (int i4 = 0; i4 < TILE / 4; ++i4) {   // packed pairs, the scalar form's rounding
                         const float4 q4 = x4[i4];
-                        v[4 * i4 + 0] = fmaf(-2.f, v[4 * i4 + 0], sqa + q4.x);
-                        v[4 * i4 + 1] = fmaf(-2.f, v[4 * i4 + 1], sqa + q4.y);
-                        v[4 * i4 + 2] = fmaf(-2.f, v[4 * i4 + 2], sqa + q4.z);
-                        v[4 * i4 + 3] = fmaf(-2.f, v[4 * i4 + 3], sqa + q4.w);
+                        const float2 a = __ffma2_rn(m2, make_float2(v[4 * i4], v[4 * i4 + 1]), __fadd2_rn(sq2, make_float2(q4.x, q4.y)));
+                        const float2 c = __ffma2_rn(m2, make_float2(v[4 * i4 + 2], v[4 * i4 + 3]), __fadd2_rn(sq2, make_float2(q4.z, q4.w)));
+                        v[4 * i4] = a.x;
+                        v[4 * i4 + 1] = a.y;
+                        v[4 * i4 + 2] = c.x;
+                        v[4 * i4 + 3] = c.y;
                     }
                 }
                 tc::fence_before_sync();
@@ -2651,21 +2657,29 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) knn_tcp_kernel(TileArgs a)
                     evaluated += TILE;
 #pragma unroll
                     for (int ch = 0; ch < TILE / 32; ++ch) {
-                        // mask of the columns under the bound: four independent 8-bit chains
+                        // columns under the bound: the sign bits of bound - distance (its rounded sign is exact),
+                        // shifted in one by one in four independent 8-bit chains
+                        const float2 h2 = make_float2(hmf, hmf), n1 = make_float2(-1.f, -1.f);
                         uint32_t mq[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) mq[i & 3] |= (v[ch * 32 + i] <= hmf ? 1u : 0u) << i;
-                        uint32_t msk = (mq[0] | mq[1]) | (mq[2] | mq[3]);
+                        for (int i = 6; i >= 0; i -= 2) {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const float* vv = v + ch * 32 + 8 * q + i;
+                                const float2 t2 = __ffma2_rn(n1, make_float2(vv[0], vv[1]), h2);
+                                mq[q] = __funnelshift_l(__float_as_uint(t2.y), mq[q], 1);
+                                mq[q] = __funnelshift_l(__float_as_uint(t2.x), mq[q], 1);
+                            }
+                        }
+                        uint32_t msk = ~(mq[0] | mq[1] << 8 | mq[2] << 16 | mq[3] << 24);
                         while (msk) {   // the full key test and the heap update
                             const int i = __ffs(msk) - 1;
                             msk &= msk - 1u;
-                            float d = 0.f;
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) d = j == i ? v[ch * 32 + j] : d;
+                            const float d = Pick<32>::get(v + ch * 32, i);
                             const int64_t cp = (int64_t)ct * TILE + ch * 32 + i;
                             const uint64_t key = ((uint64_t)__float_as_uint(fmaxf(d, 0.f)) << 32) | (uint32_t)cp;
                             if (key < heapmax && cp != p && cp >= qlo && cp < qhi) {
-                                sift_down<T2>(heap, t, 0, L, key, levels);
+                                sift_down_d<T2, TC_ARITY>(heap, t, 0, L, key, levels);
                                 heapmax = heap[t];
                             }
                         }
@@ -2744,7 +2758,7 @@ __global__ void __launch_bounds__(T2) tcp_finish_kernel(TileArgs a)
         const float sqa = ((const float*)(a.blk + (p / TILE) * BLK + tcp_img_bytes(a.kp)))[p % TILE];
         const float qn = sqrtf(sqa);
         ok = !(F16 && qn > 0.25f * kHalfClamp);
-        if (ok) ok = finalize_row_band<MP, T2>(a, a.hdump + (size_t)qs * L * T2, t, L, p, qhi - qlo, levels, bd, qn);
+        if (ok) ok = finalize_row_band<MP, T2, uint64_t, TC_ARITY>(a, a.hdump + (size_t)qs * L * T2, t, L, p, qhi - qlo, levels, bd, qn);
     }
     if (__syncthreads_or(!ok) && t == 0) {
         for (int h = 0; h < 2; ++h) {
