@@ -3223,7 +3223,7 @@ vb_status knn_run(Ctx* ctx, const float* x, int64_t n, int32_t m, const vb_knn_p
     // the tiles a radius-first or 16-bit first pass hands back are searched with compact keys
     // before the full-key search takes what is left
     // m <= 8: the warp search, also for 16-bit requests at m <= 4 that name no kernel and want no diagnostic
-    const bool warp_search = warp_search_takes(mp, p) &&
+    const bool warp_search = warp_search_takes(mp, p) && n < INT32_MAX - 4096 &&   // padded positions fit an int
                              (!tensor || (mp == 4 && p->tc_variant == VB_TC_AUTO && !a.dbg_d2));
     const bool compact_retry = (radius_first || tensor) && p->heap_keys != VB_KEYS_FULL && mp <= 16 && !warp_search;
     int launches = 0;
