@@ -8,7 +8,8 @@ from a CUDA graph recorded once per form.  Every form computes the same
 matrix (neighbour lists and L-hat bit for bit, asserted); the forms differ in
 how the kNN search gets there:
   plain_fp32        exact heap search with FP32 ALU distance tiles (the comparison the metric names)
-  fp16_tc, bf16_tc  16-bit distance tiles on the tensor cores (tcgen05.mma), FP64 rescoring
+  fp16_tc, bf16_tc  16-bit distance tiles on the tensor cores (tcgen05.mma), FP64 rescoring; at m <= 4 the
+                    autotuner may find the FP32 warp search faster for the request, and dtype says so
   learned_*         the same with each query's heap started at a radius predicted by the
                     learned network (trained beforehand on a separate draw, not timed)
   const_radius_fp32 ablation of the learned part: one global radius for every point
@@ -248,7 +249,12 @@ KNN_SEARCH_STAGES = ("knn_radius", "knn_tile", "knn_retry")   # the search prope
 
 
 def _stage_kernel(stage: str, form: str, shape: dict) -> str:
-    """The kernel that does a stage's work (the stage's other launches are small set-up passes)."""
+    """The kernel that does a stage's work (the stage's other launches are small set-up passes).
+    shape: the form's autotuned choices and the workload's m and k; at m <= 8 and k <= 128 the FP32
+    search, and at m <= 4 a 16-bit request that names no kernel, is the warp search."""
+    m, warp = shape.get("m", 128), shape.get("m", 128) <= 8 and shape.get("k", 256) <= 128
+    if stage == "knn_tile" and warp and (not form.endswith("_tc") or (m <= 4 and shape.get("tc_variant") == "auto")):
+        return "knn_warp_kernel"
     if stage == "knn_tile" and form.endswith("_tc"):
         return "knn_tcp_kernel" if shape.get("tc_variant") == "pipelined" else "knn_tc_kernel"
     return {"knn_tile": "knn_tile_kernel", "knn_retry": "knn_tile_kernel", "knn_radius": "mlp_radius_tc_kernel",
@@ -501,6 +507,9 @@ def main():
     KP = (spec.m + 15) // 16 * 16
     tensor_tflops = peaks.get("bf16_tflops", 1900.0)     # FP16 and BF16 run at the same dense rate
 
+    best_shape = dict(shapes[best], m=spec.m, k=spec.k)
+    warp_search = _stage_kernel("knn_tile", best, best_shape) == "knn_warp_kernel"
+
     def roof(stage):
         ms = stage_ms.get(stage)
         if not ms:
@@ -511,7 +520,7 @@ def main():
             return {"bound": "alu", "unit": "Gentries/s", "achieved": ach, "peak": peak, "frac": ach / peak,
                     "what": f"{G} kernel values per off-diagonal entry, {EX2_PER_ENTRY} ex2 on the SFU "
                             f"({N_SM} SM x {SFU_PER_SM_CLK}/clk x {f_mhz:.0f} MHz / {EX2_PER_ENTRY})"}
-        if stage == "knn_tile" and best.endswith("_tc"):
+        if stage == "knn_tile" and best.endswith("_tc") and not warp_search:
             ach = cand * 2 * spec.m / s / 1e12
             return {"bound": "tensor", "unit": "TFLOP/s", "achieved": ach, "peak": tensor_tflops,
                     "frac": ach / tensor_tflops,
@@ -548,7 +557,7 @@ def main():
     droof = roof(dom) or {"bound": "hbm", "achieved": None, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": None}
     droof = {kk: droof[kk] for kk in ("bound", "achieved", "peak", "unit", "frac", "what") if kk in droof}
     droof["stage"] = dom
-    droof["kernel"] = _stage_kernel(dom, best, shapes[best])
+    droof["kernel"] = _stage_kernel(dom, best, best_shape)
     droof["traffic"] = _traffic(dom, best, spec.name)
 
     sizes = np.diff(spec.cloud_ptr) if batched else np.array([spec.n])
@@ -558,7 +567,7 @@ def main():
                 "parallelism": f"replicas x{ws}", "timing": "CUDA-graph replay of the whole build per step"})
     line = {"metric": METRIC, "value": value, "unit": "points/s", "n_gpus": ws, "steps": a.steps, "warmup": a.warmup,
             "ms_per_step": 1e3 * total_s / a.steps, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": {"bf16": "bf16+f32", "fp16": "f16+f32"}.get(best.split("_")[-2], "f32"),
+            "vs_baseline": None, "dtype": "f32" if warp_search else {"bf16": "bf16+f32", "fp16": "f16+f32"}.get(best.split("_")[-2], "f32"),
             "data": "synthetic", "config": cfg,
             "forms": {f: {"ms_per_step": 1e3 * res[f]["total_s"] / a.steps,
                           "points_per_s": job_throughput(spec.n, a.steps, ws, res[f]["total_s"]),
