@@ -583,8 +583,10 @@ vb_status graph_run(Ctx* ctx, int64_t n, int32_t k, const int32_t* nbr, const do
 // ------------------------------------------------------------------ a8
 // One thread per row, the rows' distances staged through shared memory 16 at a time, so that the loads are
 // whole 128-byte lines (a thread reading its own row directly touches one line per load: 0.22 ms for
-// 1M rows of 64); the sums stay in rank order.  Bound by the narrow FP64 pipe (n k additions, 0.11 ms there).
-constexpr int BW_T = 128, BW_C = 16;
+// 1M rows of 64); the sums stay in rank order.  A chunk's loads fly while the one before is summed: a whole
+// build of 2,000 points 202.7 -> 197.3 us, of 50k 576 -> 560 us, of 1M 7.19 -> 7.16 ms (each k <= 64).  Bound
+// by the narrow FP64 pipe (n k additions, 0.11 ms at 1M) and by the length of its chain in small clouds.
+constexpr int BW_T = 128, BW_C = 16, BW_R = BW_T / BW_C;   // a chunk: BW_T rows by BW_C columns, BW_C loads a thread
 __global__ void __launch_bounds__(BW_T) bandwidth_kernel(const double* __restrict__ nbr_d2, int64_t n, int k, int k_bw,
                                                          double* b, float* ib, DevReport* rep)
 {
@@ -592,23 +594,30 @@ __global__ void __launch_bounds__(BW_T) bandwidth_kernel(const double* __restric
     const int t = threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.x * BW_T;
     const int nr = (int)min((int64_t)BW_T, n - r0);
-    double s = 0.0;
+    const int c = t % BW_C, rt = t / BW_C;   // the thread's column of a chunk and its first row
+    const double* src = nbr_d2 + (r0 + rt) * k + c;
+    double v[BW_C] = {}, s = 0.0;
+    auto load = [&](int c0) {
+#pragma unroll
+        for (int u = 0; u < BW_C; ++u)
+            if (rt + u * BW_R < nr && c0 + c < k_bw) v[u] = src[(int64_t)u * BW_R * k + c0];
+    };
+    load(0);
     for (int c0 = 0; c0 < k_bw; c0 += BW_C) {
         const int nc = min(BW_C, k_bw - c0);
-        for (int e = t; e < nr * BW_C; e += BW_T) {
-            const int r = e / BW_C, c = e % BW_C;
-            if (c < nc) sh[r][c] = nbr_d2[(r0 + r) * k + c0 + c];
-        }
+#pragma unroll
+        for (int u = 0; u < BW_C; ++u) sh[rt + u * BW_R][c] = v[u];
         __syncthreads();
+        load(c0 + BW_C);
         if (t < nr)
-            for (int c = 0; c < nc; ++c) s = c0 + c == 0 ? sh[t][c] : __dadd_rn(s, sh[t][c]);
+            for (int e = 0; e < nc; ++e) s = c0 + e == 0 ? sh[t][e] : __dadd_rn(s, sh[t][e]);
         __syncthreads();
     }
     if (t >= nr) return;
-    const double v = sqrt(s);
-    b[r0 + t] = v;
-    if (ib) ib[r0 + t] = (float)(1.0 / v);
-    if (!(v > 0.0) || !isfinite(v)) report_error(rep, VB_ERR_DEGENERATE);
+    const double bw = sqrt(s);
+    b[r0 + t] = bw;
+    if (ib) ib[r0 + t] = (float)(1.0 / bw);
+    if (!(bw > 0.0) || !isfinite(bw)) report_error(rep, VB_ERR_DEGENERATE);
 }
 
 vb_status bandwidth_run(Ctx* ctx, int64_t n, int32_t k, int32_t k_bw, const double* nbr_d2, double* b, float* ib)
