@@ -83,7 +83,7 @@ static int pad_dim(int m)
     while (mp < m) mp *= 2;
     return mp;
 }
-constexpr int PCA_D = 5;           // principal axes of the Morton key when m > 4
+constexpr int PCA_D = 5;           // principal axes of the spatial key when m > 4
 static int morton_dims(int m) { return m <= 4 ? m : PCA_D; }
 static int morton_bits(int md) { return md == 1 ? 30 : md == 2 ? 15 : md == 3 ? 10 : md == 4 ? 8 : md == 5 ? 6 : 5; }
 
@@ -3049,7 +3049,7 @@ static vb_status launch_tile(const TileArgs& a, cudaStream_t s)
     return launch_tile_m<MP, MP, K32>(a, s);
 }
 
-// a1: the spatial order of the points (Morton key on the coordinates, or on the projections on
+// a1: the spatial order of the points (Hilbert or Morton key on the coordinates, or on the projections on
 // the leading principal axes when m > 4; then the cloud id above it in a batch), the sorted
 // coordinates in FP32 and FP64, and the boxes of 64-point tiles and 64-tile super-tiles.
 // perm (sorted position -> original index) is w.val[*cur] afterwards.
