@@ -501,7 +501,8 @@ __global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn
                 }
             };
             int nlist = -1;   // tiles in the group's list (-1: none, scan the boxes)
-            float rl2 = INFINITY;   // the list holds every tile that close to the group's box (squared)
+            float rl2 = INFINITY;   // the list holds every tile that close to the group's box (squared): no
+                                    // threshold under scan is above it while there is a list
             auto scan = [&](bool two) {
                 // 32 tiles per step: the next of the list, or half of the next super-tile in reach
                 unsigned ms = 0;
@@ -575,7 +576,7 @@ __global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn
                 for (int u = 0; u < 2; ++u) {
                     if (rmode && (todo >> u & 1)) r2q[u] = __fmul_ru(a.r2[p[u]], a.r2_scale);
                     tmax[u] = fminf(pmax[u], r2q[u]);
-                    thr[u] = (todo >> u & 1) ? fminf(guess, tmax[u]) : -1.f;
+                    thr[u] = (todo >> u & 1) ? fminf(fminf(guess, tmax[u]), rl2) : -1.f;
                 }
                 int np = 0, tries = 0;
                 while (todo) {
@@ -632,8 +633,8 @@ __global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn
                         }
                         tmax[u] = fminf(pmax[u], 4.f * r2q[u]);
                         thr[u] = tmax[u];
-                        if (!(tmax[u] <= rl2)) nlist = -1;   // beyond the list's reach
                     }
+                    if (!(fmaxf(thr[0], thr[1]) <= rl2)) nlist = -1;   // beyond the list's reach
                 }
                 return true;
             };
@@ -681,11 +682,13 @@ __global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn
                     // ---- the others, two at a time
                     const bool two = i + 1 < s1;
                     load_query(1, two ? i + 1 : i);
-                    pm[0] = fminf(bound(0), rl2);
-                    pm[1] = fminf(bound(1), rl2);
+                    pm[0] = bound(0);
+                    pm[1] = bound(1);
                     if (two) todo = 3;
                 }
-                // ---- the group's candidate tiles: boxes within the query's bound + the reach of the rest of the group
+                // ---- the group's candidate tiles: boxes within the queries' bound + the reach of the rest of the group.
+                // A later query with a larger bound (a radius guess proves nothing about its neighbours') starts at the
+                // list's reach; if it needs more, the boxes are scanned and the next pair makes a new list.
                 if (nlist < 0 && !norelist && s1 - i > 3) {
                     const bool mine = lane < s1 - i;
                     float4 v[MP / 4];
@@ -708,7 +711,10 @@ __global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn
                             bhi[r] = fmaxf(bhi[r], __shfl_xor_sync(0xffffffffu, bhi[r], o));
                         }
                     }
-                    const float base = fminf(pm[0], rmode ? __fmul_ru(a.r2[i], a.r2_scale) : INFINITY);
+                    // the larger of the thresholds that the queries at hand may start with: guesses differ
+                    float base = fminf(pm[0], rmode ? __fmul_ru(a.r2[i], a.r2_scale) : INFINITY);
+                    if (todo == 3)
+                        base = fmaxf(base, fminf(pm[1], rmode ? __fmul_ru(a.r2[i + 1], a.r2_scale) : INFINITY));
                     const float rl = __fadd_ru(__fsqrt_ru(base), __fsqrt_ru(__fmul_ru(reach, 1.00001f)));
                     const float near2 = __fmul_ru(__fmul_ru(rl, rl), 1.00001f);
                     auto near = [&](const float* lo, const float* hi, int idx) {
