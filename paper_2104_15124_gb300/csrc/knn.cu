@@ -3130,9 +3130,10 @@ static vb_status order_points(Ctx* ctx, const float* x, int64_t n, int32_t m, co
                                                       w.hist, nblk, items, fused);
         cur ^= 1;
     };
-    // keys of md * bits bits; below 2^18 points the lowest eight would only order points inside cells far
-    // smaller than a tile
-    for (int shift = n < (1 << 18) && md * bits >= 30 ? 8 : 0; shift < md * bits; shift += 8) radix_pass(shift);
+    // all md * bits bits: the cells divide the box of all points, so with tails, outliers or tight clusters the
+    // low bits are what separates most of them (100k points with 1 % of them 30 times farther out, m = 3, k = 48:
+    // 20 tiles a query and 0.96 ms, without the lowest byte 186 and 2.4 ms; 17 us on 50k near-uniform points)
+    for (int shift = 0; shift < md * bits; shift += 8) radix_pass(shift);
     if (cl.B > 1) {
         // stable passes on the cloud id: (cloud, Morton) order, so cloud b occupies the sorted
         // positions [ptr[b], ptr[b + 1]), the same range as its points in the input
