@@ -3146,6 +3146,7 @@ static vb_status order_points(Ctx* ctx, const float* x, int64_t n, int32_t m, co
     tile_box_kernel<<<(unsigned)((ntiles * 32 + 255) / 256), 256, 0, s>>>(w.xs, n, ntiles, m, mp, w.tlo, w.thi);
     super_box_kernel<<<(unsigned)(((ntiles + TILE - 1) / TILE * 32 + 255) / 256), 256, 0, s>>>(w.tlo, w.thi, ntiles, mp,
                                                                                               w.slo, w.shi);
+    ctx->launches += 6;   // bbox init, bbox, keys, gather, boxes, super-tile boxes (the others counted above)
     *perm_out = perm;
     return last_launch();
 }
@@ -3388,7 +3389,7 @@ vb_status knn_run(Ctx* ctx, const float* x, int64_t n, int32_t m, const vb_knn_p
     ctx->launches += launches;
     knn_fallback_kernel<<<152, FB_THREADS, 0, s>>>(x, n, m, p->k, w.fb_list, w.fb_count, cl, nbr, nbr_d2);
     mark(ctx, VB_STAGE_KNN_FALLBACK, 1);
-    ctx->launches += 8;   // order: bbox init, bbox, Morton keys, gather, boxes, super-tile boxes (radix passes counted above); search; fallback
+    ctx->launches += 2;   // exact search, fallback
     return last_launch();
 }
 
