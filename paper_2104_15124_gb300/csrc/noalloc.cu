@@ -7,7 +7,7 @@
 // and embeddings that run under a fixed device-memory budget.  They still
 // pass their inputs and outputs; only the scratch moves into the library.
 //
-// The scratch (z = x / S as a pair of floats and S, a 16-byte record per row) lives in
+// The scratch (z = x / S and S, a 16-byte record per row) lives in
 // the file-scope array g_lap_scratch, sized for VB_NOALLOC_MAX_N rows; every
 // GPU that loads libvb holds it (about 16.8 MB) until the process exits.  Host
 // code cannot use the array's name as a device address, so the first call on

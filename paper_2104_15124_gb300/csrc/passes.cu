@@ -1040,14 +1040,19 @@ __global__ void __launch_bounds__(kRowThreads) spmv_plain_kernel(const int64_t* 
 }
 
 // What an entry of the difference form gathers from its column j, in one 16-byte record: z = x / S
-// as an unevaluated pair of floats, and S.
+// as an unevaluated pair of floats, and S.  A z that the pair cannot hold to 48 bits (beyond 2^126 or below
+// 2^-80 in magnitude) is kept in FP64 in the pair's place, and the fourth word says so.
 __global__ void lap_prep_kernel(const float* __restrict__ x, const double* __restrict__ S, int64_t n, float4* rec)
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) {
-        const double si = S[i], z = (double)x[i] / si;
-        const float h = (float)z;
-        rec[i] = make_float4(h, isfinite(h) ? (float)(z - (double)h) : 0.f, (float)si, 0.f);
+        const double si = S[i], z = (double)x[i] / si, az = fabs(z);
+        if (az == 0.0 || (az >= 0x1p-80 && az < 0x1p126)) {
+            const float h = (float)z;
+            rec[i] = make_float4(h, (float)(z - (double)h), (float)si, 0.f);
+        } else {
+            rec[i] = make_float4(__int_as_float(__double2loint(z)), __int_as_float(__double2hiint(z)), (float)si, 1.f);
+        }
     }
 }
 
@@ -1057,13 +1062,18 @@ __device__ __forceinline__ float pair_diff(const float4& a, const float4& b)
 {
     const float d = __fsub_rn(a.x, b.x), v = __fsub_rn(d, a.x);
     const float err = __fsub_rn(__fsub_rn(a.x, __fsub_rn(d, v)), __fadd_rn(b.x, v));
-    const float r = __fadd_rn(d, __fadd_rn(err, __fsub_rn(a.y, b.y)));
-    return isfinite(d) ? r : d;
+    return __fadd_rn(d, __fadd_rn(err, __fsub_rn(a.y, b.y)));
 }
+// The same in FP64, for records outside the pairs' range (out of line, as they are rare).
+__device__ __forceinline__ double rec_z(const float4& r)
+{
+    return r.w != 0.f ? __hiloint2double(__float_as_int(r.y), __float_as_int(r.x)) : (double)r.x + (double)r.y;
+}
+__device__ __noinline__ float wide_diff(float4 a, float4 b) { return (float)(rec_z(a) - rec_z(b)); }
 
 // y_i = alpha sum_{j != i} val_ij S_j (z_j - z_i) + beta y_i, z = x / S.  The differences are taken on
 // float pairs, so smooth vectors keep their accuracy as with FP64 differences, without an
-// operation of the narrow FP64 pipe per entry.  Eight lanes a row and a quad of entries a lane, as in
+// operation of the narrow FP64 pipe per entry (an FP64 z in the record: 0.45 ms).  Eight lanes a row and a quad of entries a lane, as in
 // the row passes.  Bound by the gathers, a 32-byte sector of L2 per entry: 0.61 ms with a warp per row and
 // two gathers (FP64 z, S) per entry, 0.33 ms so, on 1M torus points (73M entries).
 __global__ void __launch_bounds__(kRowThreads) spmv_lap_kernel(const int64_t* __restrict__ row_ptr,
@@ -1086,11 +1096,14 @@ __global__ void __launch_bounds__(kRowThreads) spmv_lap_kernel(const int64_t* __
             float4 rj[UNR];
             load_quad(col, val, vec, e0, rb, re, jj, vv);
 #pragma unroll
-            for (int u = 0; u < UNR; ++u)
-                if (jj[u] >= 0) rj[u] = rec[jj[u]];
+            for (int u = 0; u < UNR; ++u) rj[u] = jj[u] >= 0 ? rec[jj[u]] : make_float4(0.f, 0.f, 0.f, 0.f);
+            const bool wide = ri.w + ((rj[0].w + rj[1].w) + (rj[2].w + rj[3].w)) != 0.f;
 #pragma unroll
-            for (int u = 0; u < UNR; ++u)
-                if (jj[u] >= 0 && jj[u] != i) s[u] = fmaf(vv[u] * rj[u].z, pair_diff(rj[u], ri), s[u]);
+            for (int u = 0; u < UNR; ++u) {
+                float d = pair_diff(rj[u], ri);
+                if (wide) d = wide_diff(rj[u], ri);
+                if (jj[u] >= 0 && jj[u] != i) s[u] = fmaf(vv[u] * rj[u].z, d, s[u]);
+            }
         }
         const double tot = (double)RowGroup<LPR>::sum((s[0] + s[1]) + (s[2] + s[3]));
         if (ok && it.sub == 0) y[i] = (float)((double)alpha * tot + (beta != 0.f ? (double)beta * y[i] : 0.0));
