@@ -584,9 +584,11 @@ vb_status graph_run(Ctx* ctx, int64_t n, int32_t k, const int32_t* nbr, const do
 // One thread per row, the rows' distances staged through shared memory 16 at a time, so that the loads are
 // whole 128-byte lines (a thread reading its own row directly touches one line per load: 0.22 ms for
 // 1M rows of 64); the sums stay in rank order.  A chunk's loads fly while the one before is summed: a whole
-// build of 2,000 points 202.7 -> 197.3 us, of 50k 576 -> 560 us, of 1M 7.19 -> 7.16 ms (each k <= 64).  Bound
-// by the narrow FP64 pipe (n k additions, 0.11 ms at 1M) and by the length of its chain in small clouds.
-constexpr int BW_T = 128, BW_C = 16, BW_R = BW_T / BW_C;   // a chunk: BW_T rows by BW_C columns, BW_C loads a thread
+// build of 2,000 points 202.7 -> 197.3 us, of 50k 576 -> 560 us, of 1M 7.19 -> 7.16 ms (each k <= 64).  Blocks of
+// 64 rows, so that 20,000 points fill the chip (k = 200: 25 us with 128 rows, 21 us with a thread reading its row,
+// 19 us so; 100k, k = 32: 15 -> 13 us).  Bound by the narrow FP64 pipe (n k additions, 0.11 ms at 1M) and by the
+// length of its chain in small clouds.
+constexpr int BW_T = 64, BW_C = 16, BW_R = BW_T / BW_C;   // a chunk: BW_T rows by BW_C columns, BW_C loads a thread
 __global__ void __launch_bounds__(BW_T) bandwidth_kernel(const double* __restrict__ nbr_d2, int64_t n, int k, int k_bw,
                                                          double* b, float* ib, DevReport* rep)
 {
