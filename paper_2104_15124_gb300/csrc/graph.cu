@@ -151,7 +151,8 @@ struct GraphWs {
     int32_t* rev_col;  // n k: those beyond RBUCKET, entry e of row j at row_ptr[j] - j (1 + k) + e
     float* rev_d2;     // n k
     int32_t* big;      // n rows for the block path
-    int32_t* nbig;     // [0] rows for the block path, [1] entries beyond RBUCKET
+    int32_t* nbig;     // rows for the block path
+    unsigned long long* nover;   // entries beyond RBUCKET (n k of them at most: they can pass 2^32)
     int4* over;        // OVER_CAP of those: (i, j, distance bits, -)
     void* scan;        // scan_ws_bytes(n)
 };
@@ -168,7 +169,8 @@ static size_t graph_plan(Carve& c, int64_t n, int32_t k, GraphWs* w)
     t.rev_col = c.take<int32_t>(n * (int64_t)k);
     t.rev_d2 = c.take<float>(n * (int64_t)k);
     t.big = c.take<int32_t>(n);
-    t.nbig = c.take<int32_t>(2);
+    t.nbig = c.take<int32_t>(1);
+    t.nover = c.take<unsigned long long>(1);
     t.over = c.take<int4>(OVER_CAP);
     t.scan = c.take<char>(scan_ws_bytes(n));
     if (w) *w = t;
@@ -225,10 +227,13 @@ constexpr int SORT_WARPS = 4;
 // test below reads at random stays in L2, where the lists themselves (12 k bytes per point)
 // do not.
 __global__ void kth_kernel(const int32_t* __restrict__ nbr, const double* __restrict__ nbr_d2, int64_t n, int k,
-                           Kth* kth, int32_t* rcnt, int32_t* fill, int32_t* nbig)
+                           Kth* kth, int32_t* rcnt, int32_t* fill, int32_t* nbig, unsigned long long* nover)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < 2) nbig[i] = 0;
+    if (i == 0) {
+        *nbig = 0;
+        *nover = 0;
+    }
     if (i >= n) return;
     rcnt[i] = 0;
     fill[i] = 0;
@@ -251,7 +256,7 @@ __global__ void kth_kernel(const int32_t* __restrict__ nbr, const double* __rest
 // else an entry's place is the number of columns below its own: every column is broadcast to the warp
 // once and each lane counts for the KL entries it holds.
 __device__ __forceinline__ float own_entry(int64_t i, int32_t j, double d, int k, const Kth* __restrict__ kth,
-                                           int32_t* rcnt, int2* bucket, int32_t* nover, int4* over)
+                                           int32_t* rcnt, int2* bucket, unsigned long long* nover, int4* over)
 {
     const Kth q = kth[j];
     const float f = (float)d;
@@ -261,7 +266,7 @@ __device__ __forceinline__ float own_entry(int64_t i, int32_t j, double d, int k
         bucket[(int64_t)j * RBUCKET + slot] = make_int2((int32_t)i, __float_as_int(f));
         return f;
     }
-    const int at = atomicAdd(nover, 1);
+    const unsigned long long at = atomicAdd(nover, 1ull);
     if (at < OVER_CAP) over[at] = make_int4((int32_t)i, j, __float_as_int(f), 0);
     return -f;
 }
@@ -271,7 +276,7 @@ __global__ void __launch_bounds__(SORT_WARPS * 32) own_sort_kernel(const int32_t
                                                                     const double* __restrict__ nbr_d2, int64_t n,
                                                                     int k, int32_t* own_col, float* own_d2,
                                                                     const Kth* __restrict__ kth, int32_t* rcnt,
-                                                                    int2* bucket, int32_t* nover, int4* over)
+                                                                    int2* bucket, unsigned long long* nover, int4* over)
 {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int64_t i = (int64_t)blockIdx.x * SORT_WARPS + w; i < n; i += (int64_t)gridDim.x * SORT_WARPS) {
@@ -330,12 +335,12 @@ __global__ void __launch_bounds__(SORT_WARPS * 32) own_sort_kernel(const int32_t
 // scattered behind row_ptr.
 __global__ void reverse_kernel(const int32_t* __restrict__ own_col, const float* __restrict__ own_d2, int64_t n, int k,
                                const int64_t* __restrict__ row_ptr, int32_t* fill, int32_t* rev_col, float* rev_d2,
-                               const int32_t* __restrict__ nover, const int4* __restrict__ over)
+                               const unsigned long long* __restrict__ nover, const int4* __restrict__ over)
 {
-    const int no = *nover;
+    const unsigned long long no = *nover;
     if (no == 0) return;
     if (no <= OVER_CAP) {
-        for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < no; e += gridDim.x * blockDim.x) {
+        for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < (int)no; e += gridDim.x * blockDim.x) {
             const int4 v = over[e];
             const int64_t off = row_ptr[v.y] - (int64_t)v.y * (1 + k) + RBUCKET + atomicAdd(&fill[v.y], 1);
             rev_col[off] = v.x;
@@ -536,14 +541,13 @@ vb_status graph_run(Ctx* ctx, int64_t n, int32_t k, const int32_t* nbr, const do
     if (!ws || ws_bytes < need) return VB_ERR_WORKSPACE;
     cudaStream_t s = ctx->stream;
     mark(ctx, VB_STAGE_GRAPH, 0);
-    int32_t* nover = w.nbig + 1;
-    kth_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(nbr, nbr_d2, n, k, w.kth, w.rcnt, w.fill, w.nbig);
+    kth_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(nbr, nbr_d2, n, k, w.kth, w.rcnt, w.fill, w.nbig, w.nover);
     // sorted by keys of a column and a position while those fit 32 bits, else ranked by counting
     const int pb = k <= 32 ? 5 : k <= 64 ? 6 : 7;
     const bool keys = k <= 128 && n <= (int64_t)1 << (32 - pb);
 #define VB_OWN(KL, SORT)                                                                                            \
     own_sort_kernel<KL, SORT><<<152 * 16, SORT_WARPS * 32, 0, s>>>(nbr, nbr_d2, n, k, w.own_col, w.own_d2, w.kth,     \
-                                                                w.rcnt, w.bucket, nover, w.over)
+                                                                w.rcnt, w.bucket, w.nover, w.over)
     if (k <= 32) {
         if (keys) VB_OWN(1, true); else VB_OWN(1, false);
     } else if (k <= 64) {
@@ -556,7 +560,7 @@ vb_status graph_run(Ctx* ctx, int64_t n, int32_t k, const int32_t* nbr, const do
 #undef VB_OWN
     vb_status st = scan_counts(s, w.rcnt, n, row_ptr, w.scan, 1 + k);
     if (st != VB_OK) return st;
-    reverse_kernel<<<152 * 8, 256, 0, s>>>(w.own_col, w.own_d2, n, k, row_ptr, w.fill, w.rev_col, w.rev_d2, nover, w.over);
+    reverse_kernel<<<152 * 8, 256, 0, s>>>(w.own_col, w.own_d2, n, k, row_ptr, w.fill, w.rev_col, w.rev_d2, w.nover, w.over);
 #define VB_MERGE(KL)                                                                                                 \
     merge_kernel<KL><<<152 * 16, SORT_WARPS * 32, 0, s>>>(row_ptr, n, k, w.own_col, w.own_d2, w.bucket, w.rev_col,      \
                                                          w.rev_d2, col, ed2, cap, w.big, w.nbig, nnz_dev, ctx->rep)
