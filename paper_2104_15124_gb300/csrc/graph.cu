@@ -133,7 +133,11 @@ vb_status scan_counts(cudaStream_t s, const int32_t* counts, int64_t n, int64_t*
 // which merges the three sorted sets with no duplicates left to remove.
 constexpr int RCAP = 256;           // warp path: reverse entries per row held in shared memory
 constexpr int OWN_CAP = 256;        // longest kNN list (k + margin <= 256)
-constexpr int RBUCKET = 32;         // reverse entries a row takes without the second pass
+// Reverse entries a row takes without the second pass.  Clouds in many dimensions have hubs: 100k points in R^16,
+// k = 64 and 128, take 0.42 and 1.12 ms with 32, 0.38 and 1.02 ms with 64 (without buckets 0.36 and 0.99 ms, but
+// 1.49 against 1.04 ms on 1M torus points, whose rows have few reverse entries).
+constexpr int RBUCKET = 64;
+constexpr int RSMALL = 32;          // reverse entries that a warp merges without sorting them
 constexpr int OVER_CAP = 1 << 16;   // entries beyond the buckets that are listed (more: every list is scanned)
 
 struct Kth {
@@ -497,7 +501,7 @@ __global__ void __launch_bounds__(SORT_WARPS * 32) merge_kernel(const int64_t* _
             }
             continue;
         }
-        if (r <= RBUCKET)
+        if (r <= RSMALL)
             merge_row_small<KL>(j, k, r, row_ptr, own_col, own_d2, bucket, col, ed2, lane, ocs[w]);
         else
             merge_row(j, k, r, buf[w], row_ptr, own_col, own_d2, bucket, rev_col, rev_d2, col, ed2, lane, 32, true, ocs[w]);
