@@ -391,7 +391,8 @@ vb_status radius_sweep_run(Ctx* ctx, const float* x, int64_t n, int32_t m, const
     cudaStream_t s = ctx->stream;
     const unsigned grid = (unsigned)std::min<int64_t>(r.o.ntiles, kRadiusBlocks);
     unsigned nblk = grid;
-    if (G == RG57 && dxi == 0.25) {
+    // (2^xi, its inverse and tau 2^xi are normal numbers there; beyond, the general pass divides as before)
+    if (G == RG57 && dxi == 0.25 && xi_lo >= -960.0 && xi_hi <= 960.0) {
         SweepGrid sg;
         for (int g = 0; g < G; ++g) {
             double x = tau * gv.v[g];
