@@ -164,7 +164,26 @@ __global__ void __launch_bounds__(GT) mlp_grad_kernel(MlpK k, const float* __res
     const float b3 = __bfloat162float(k.wb[o.b3]);
     const int s = t / 8, g = t % 8;              // sample and thread of it
     const int j0 = (t / 16) * 4, i0 = (t % 16) * 4;   // the patch of W2's gradient
-    float a2[4][4] = {}, a1[4] = {}, av = 0.f, lsum = 0.f;
+    // sums of the last 128 samples, and of those before: a block takes 6,600 samples of a million, and one running
+    // FP32 sum over them would round as often
+    float a2[4][4] = {}, a1[4] = {}, av = 0.f, lsum = 0.f, t2[4][4] = {}, t1[4] = {}, tv = 0.f, tl = 0.f;
+    int held = 0;
+    auto fold = [&]() {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                t2[a][b] += a2[a][b];
+                a2[a][b] = 0.f;
+            }
+            t1[a] += a1[a];
+            a1[a] = 0.f;
+        }
+        tv += av;
+        tl += lsum;
+        av = lsum = 0.f;
+        held = 0;
+    };
     for (int64_t base = r0 + (int64_t)blockIdx.x * GS; base < r1; base += (int64_t)gridDim.x * GS) {
         const int64_t row = base + s;
         const bool ok = row < r1;
@@ -258,20 +277,22 @@ __global__ void __launch_bounds__(GT) mlp_grad_kernel(MlpK k, const float* __res
             for (int q = 0; q < GS; ++q) av = fmaf(sdo[q], sh2[q * GLD + j], av);
         else if (t == 3 * H)
             for (int q = 0; q < GS; ++q) av += sdo[q];
+        if (++held == 128 / GS) fold();
     }
+    fold();
     float* pb = part + (int64_t)blockIdx.x * (P + 1);
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) pb[o.w2 + (j0 + a) * H + i0 + b] = a2[a][b];
+        for (int b = 0; b < 4; ++b) pb[o.w2 + (j0 + a) * H + i0 + b] = t2[a][b];
 #pragma unroll
     for (int q4 = 0; q4 < 4; ++q4)
-        if (t + q4 * GT < H * in) pb[o.w1 + t + q4 * GT] = a1[q4];
-    if (t < H) pb[o.b1 + t] = av;
-    else if (t < 2 * H) pb[o.b2 + t - H] = av;
-    else if (t < 3 * H) pb[o.w3 + t - 2 * H] = av;
-    else if (t == 3 * H) pb[o.b3] = av;
-    if (g == 0) slo[s] = lsum;
+        if (t + q4 * GT < H * in) pb[o.w1 + t + q4 * GT] = t1[q4];
+    if (t < H) pb[o.b1 + t] = tv;
+    else if (t < 2 * H) pb[o.b2 + t - H] = tv;
+    else if (t < 3 * H) pb[o.w3 + t - 2 * H] = tv;
+    else if (t == 3 * H) pb[o.b3] = tv;
+    if (g == 0) slo[s] = tl;
     __syncthreads();
     if (t == 0) {
         float l = 0.f;
