@@ -58,7 +58,8 @@ struct KnnWs {
     float* shi;
     int* fb_list;         // n
     int* fb_count;        // [0] fallback rows, [1] next query tile, [2] next failed tile, [3] failed tiles,
-                          // [4] next tile of the second list, [5] tiles in it
+                          // [4] next tile of the second list, [5] tiles in it,
+                          // [6] groups counted by the warp search, [7] tiles a query summed over them
     float* r2;            // n (radius search: squared radius bound per sorted point)
     int* fail_flag;       // 2 ntiles: flags of radius passes 1 and 2
     int* fail_list;       // 2 ntiles: tiles left by passes 1 and 2
@@ -3217,6 +3218,7 @@ vb_status knn_run(Ctx* ctx, const float* x, int64_t n, int32_t m, const vb_knn_p
     a.cert_factor = 1.0 - 2.0 * (double)(m + 2) * 5.9604644775390625e-8;
     a.nbr = nbr; a.nbr_d2 = nbr_d2; a.fb_list = w.fb_list; a.fb_count = w.fb_count; a.rep = ctx->rep;
     a.work = w.fb_count + 1;
+    a.reach = w.fb_count + 6;
     a.cl = cl;
     a.dbg_d2 = p->dbg_idx ? p->dbg_d2 : nullptr;
     a.dbg_idx = p->dbg_idx;

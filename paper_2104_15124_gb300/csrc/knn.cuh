@@ -57,6 +57,7 @@ struct TileArgs {
     int* fail_flag;         // radius search: per query tile, set once it joins fail_list
     int* fail_list;
     int* fail_count;
+    int* reach;             // warp search: groups counted, tiles a query summed over them
     Clouds cl;              // batched build: queries only take candidates from their own cloud
     DevReport* rep;
     // pipelined 16-bit search

@@ -45,6 +45,15 @@ constexpr int WS_WARPS = 4;      // warps per CTA; groups of 16 points then fill
 constexpr int WS_LIST = 256;     // candidate tiles a group's list holds (beyond it the boxes are rescanned per pair)
 constexpr int WS_MAX_G = 16;     // points per group at most
 
+// Where a query reaches most of a large cloud, every pair of queries loads the whole cloud from L2, and the
+// tiled search, which loads it once for 64 queries, is the faster one (100k Gaussian points in R^8, k = 48:
+// 1,680 tiles a query, 20 against 12 ms; 300k points of Student's t, 2 degrees, in R^4, 47 against 40 ms; at about
+// 750 they are level, in 2 to 8 dimensions).  So the groups
+// of the first WS_SAMPLE blocks, which lie all over the cloud, count the tiles a query that their first three
+// queries take, and once the mean of WS_REACH_MIN groups is above WS_REACH, the groups that have not finished
+// leave their tiles to it (13.8 and 45 ms with what was begun; clouds that stay pay 0.8 % for the counting).
+constexpr int WS_REACH = 750, WS_REACH_MIN = 256, WS_SAMPLE = 256;
+
 // Every lane keeps its own list of the candidates it found: ROWS entries, entry r of lane l at
 // [r][l].  About 1.4 k / 32 are used; a lane about to run out has the whole list cut (ws_tighten).
 // NS: sorted ranks kept for the rescoring (k <= 32 KB).  SB: bits of a list slot (r * 32 + l) in a key.
@@ -339,7 +348,8 @@ __device__ __forceinline__ void ws_append(uint32_t& at, float d, float thr, uint
 }
 
 template <int MP, int MR, int KB>
-__global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn_warp_kernel(const __grid_constant__ TileArgs a, int G)
+__global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn_warp_kernel(const __grid_constant__ TileArgs a, int G,
+                                                                                              unsigned sample)
 {
     using Cfg = WsCfg<KB>;
     constexpr int ROWS = Cfg::ROWS, NS = Cfg::NS, SB = Cfg::SB;
@@ -358,13 +368,23 @@ __global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn
     __syncthreads();
 
     const int n = (int)a.n, k = a.k;
-    const int64_t g64 = ((int64_t)blockIdx.x * WS_WARPS + warp) * G;
+    // the first WS_SAMPLE blocks take every `sample`-th block of the cloud, the others what lies between (0: in order)
+    unsigned blk = blockIdx.x;
+    if (blk < sample * WS_SAMPLE)
+        blk = blk < WS_SAMPLE ? blk * sample : blk - WS_SAMPLE + (blk - WS_SAMPLE) / (sample - 1u) + 1u;
+    const int64_t g64 = ((int64_t)blk * WS_WARPS + warp) * G;
     unsigned tests = 0;   // candidate tiles x queries scanned
     if (g64 < n) {
         const int gp0 = (int)g64, gp1 = min(n, gp0 + G);
         const int own = gp0 / TILE;
         const bool rmode = a.r2 != nullptr;
-        bool dead = false;
+        // do the groups counted so far say that the tiled search is the faster one?
+        auto wide = [&]() {
+            const int v = lane < 2 ? *(volatile int*)(a.reach + lane) : 0;
+            const int c = __shfl_sync(0xffffffffu, v, 0);
+            return c >= WS_REACH_MIN && __shfl_sync(0xffffffffu, v, 1) / c > WS_REACH;
+        };
+        bool dead = sample && wide();
         for (int s0 = gp0; s0 < gp1 && !dead;) {
             // the group's points of one cloud
             int qlo = 0, qhi = n;
@@ -759,6 +779,9 @@ __global__ void __launch_bounds__(WS_WARPS * 32, KB <= 2 && MP == 4 ? 6 : 4) knn
                 dead = !settle(todo, pm, i == s0 ? INFINITY : 1.3f * pd);
                 if (nlist < 0) rl2 = INFINITY;
                 i += todo == 3 ? 2 : 1;
+                if (sample && tests > (unsigned)(WS_REACH * (i - s0)) && wide()) dead = true;
+                if (i - s0 == 3 && blockIdx.x < WS_SAMPLE && sample && lane < 2)
+                    atomicAdd(a.reach + lane, lane == 0 ? 1 : (int)min(tests / 3, 65535u));
             }
             s0 = s1;
         }
@@ -790,7 +813,11 @@ static vb_status launch_ws(const TileArgs& a, cudaStream_t s)
     int G = 1;
     while (G < WS_MAX_G && a.n / (2 * G) >= 152 * 32) G *= 2;
     const int64_t groups = (a.n + G - 1) / G;
-    knn_warp_kernel<MP, MR, KB><<<(unsigned)((groups + WS_WARPS - 1) / WS_WARPS), WS_WARPS * 32, sm, s>>>(a, G);
+    const int64_t blocks = (groups + WS_WARPS - 1) / WS_WARPS;
+    // a cloud in which a query can reach that many tiles (a batch by its mean cloud)
+    const bool large = a.n / a.cl.B > (int64_t)WS_REACH * TILE && blocks >= 2 * WS_SAMPLE;
+    const unsigned sample = large ? (unsigned)(blocks / WS_SAMPLE) : 0u;
+    knn_warp_kernel<MP, MR, KB><<<(unsigned)blocks, WS_WARPS * 32, sm, s>>>(a, G, sample);
     return last_launch();
 }
 
