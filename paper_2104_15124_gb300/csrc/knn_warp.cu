@@ -48,10 +48,10 @@ constexpr int WS_MAX_G = 16;     // points per group at most
 // Where a query reaches most of a large cloud, every pair of queries loads the whole cloud from L2, and the
 // tiled search, which loads it once for 64 queries, is the faster one (100k Gaussian points in R^8, k = 48:
 // 1,680 tiles a query, 20 against 12 ms; 300k points of Student's t, 2 degrees, in R^4, 47 against 40 ms; at about
-// 750 they are level, in 2 to 8 dimensions).  So the groups
-// of the first WS_SAMPLE blocks, which lie all over the cloud, count the tiles a query that their first three
-// queries take, and once the mean of WS_REACH_MIN groups is above WS_REACH, the groups that have not finished
-// leave their tiles to it (13.8 and 45 ms with what was begun; clouds that stay pay 0.8 % for the counting).
+// 750 they are level, in 2 to 8 dimensions).  So the groups of the first WS_SAMPLE blocks, which lie all over
+// the cloud, count the tiles a query that their first three queries take, and once the mean of WS_REACH_MIN
+// groups is above WS_REACH, the groups that have not finished leave their tiles to it (13.8 and 45 ms with what
+// was begun; clouds that stay pay 0.8 % for the counting).
 constexpr int WS_REACH = 750, WS_REACH_MIN = 256, WS_SAMPLE = 256;
 
 // Every lane keeps its own list of the candidates it found: ROWS entries, entry r of lane l at
@@ -808,8 +808,9 @@ static vb_status launch_ws(const TileArgs& a, cudaStream_t s)
             return VB_ERR_CUDA;
         attr_set[dev & 15] = true;
     }
-    // points per warp: as many as leave every SM 32 warps (a longer group shares its first query's
-    // seeds and the tile list among more queries; a short cloud needs the warps)
+    // points per warp: as many as leave the grid 32 warps for every SM, of which 24 are resident (16 with 8-wide rows
+    // or k > 64).  A longer group shares its first query's seeds and the tile list among more queries; a short
+    // cloud needs the warps.
     int G = 1;
     while (G < WS_MAX_G && a.n / (2 * G) >= 152 * 32) G *= 2;
     const int64_t groups = (a.n + G - 1) / G;
