@@ -77,7 +77,7 @@ typedef struct {
     int64_t knn_heap_levels;    /* heap levels walked by the kNN selection (inserts and final sort) */
     int64_t knn_tiles_staged;   /* candidate tiles staged in shared memory by the kNN search */
     int64_t knn_insert_rounds;  /* per-query insertion rounds executed by the kNN search */
-    int64_t knn_retry_tiles;    /* query tiles the radius-first search handed back to the exact search */
+    int64_t knn_retry_tiles;    /* query tiles the first search handed on to the exact tiled search */
     int64_t knn_rows_short;     /* rows with fewer than k candidates kept (radius too small) */
     int64_t knn_rows_long_run;  /* rows whose FP32/16-bit ties or error band exceeded the exact-order buffer */
     int64_t knn_rows_uncertified; /* rows whose k-th FP64 distance did not clear the certificate bound */
@@ -125,7 +125,8 @@ vb_status vb_profile_read(vb_ctx* ctx, float* ms, int64_t* launches);
  * first; in the pipelined 16-bit search, also balls about the box centres) and
  * keeps the nearest FP32 (or 16-bit) candidates per row.  At m <= 8 and k <= 128
  * one warp searches each pair of points and k + margin bounds the candidates that
- * it rescores; otherwise one thread searches each point and keeps k + margin;
+ * it rescores; otherwise, and in large clouds where a query reaches most tiles,
+ * one thread searches each point and keeps k + margin;
  * an FP64 rescoring with a proven FP32 error bound certifies every row, and
  * rows that fail it are recomputed by an exact FP64 radix selection.  The
  * output is therefore exact, identical to a brute-force FP64 search. */

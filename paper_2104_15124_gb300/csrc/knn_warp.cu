@@ -27,11 +27,11 @@
 //              k-th FP64 distance lies below the smallest FP64 distance that a candidate left out can
 //              have (the next key's bucket edge, or the threshold, less the FP32 error band).
 // A query that cannot be settled (ties across the list's end, overflow) sends its 64-point tile to
-// the tiled search with full keys.
+// the tiled search with full keys; so does a large cloud in which queries reach most tiles (WS_REACH below).
 //
-// Bound: instruction issue and the latency of dependent steps (about 1,600 warp instructions per
+// Bound: instruction issue and the latency of dependent steps (about 1,800 warp instructions per
 // query, 24 warps per SM; the FP64 rescoring keeps the FP64 pipe 30 % busy).  Measured against the
-// tiled FP32 search, identical lists: 1M torus points (m = 4, k = 64) 6.51 -> 2.98 ms, 50k sphere
+// tiled FP32 search, identical lists: 1M torus points (m = 4, k = 64) 6.51 -> 3.11 ms, 50k sphere
 // points 0.51 -> 0.17 ms, 2,000 circle points 0.150 -> 0.012 ms, 20,011 Gaussian points in R^8
 // (k = 48) 3.97 -> 1.23 ms (there every tile overflowed the compact keys' visit table and was
 // searched twice); the staged BF16 search with a learned radius took 7.08 ms on the torus.
